@@ -5,7 +5,8 @@
 //   quantize_tiles_kernel permute, unsigned codes, pack            (steps 1-2)
 //   quantize_fused_kernel per-tensor scale, codes and pack in one pass (steps 1-2)
 //   weight_absmax_kernel  per-(tensor, group) max |w|             (step 1)
-//   pack_weights_kernel   per-(row, group) scale, Eq. (1) codes, pack (steps 1, 3)
+//   pack_weights_kernel   per-(row, group) scale, Eq. (1) codes, pack (steps 1, 3), for rows
+//                         too long for pack_rows.cu
 //
 // All are HBM-streaming kernels: rows are read with 16-byte loads where the
 // alignment allows, the permutation gather happens in shared memory, and one

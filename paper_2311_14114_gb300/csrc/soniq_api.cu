@@ -334,7 +334,10 @@ soniq_status soniq_pack_weights(const soniq_layout* L, const float* W, int32_t N
         cudaError_t e = launch_weight_absmax(geo, L->perm, W, N, s_w, s);
         if (e != cudaSuccess) return cuda_status(e);
     }
-    return cuda_status(launch_pack_weights(geo, L->perm, W, N, scale_mode == SONIQ_SCALE_PER_ROW, Wp, s_w, s));
+    const int32_t per_row = scale_mode == SONIQ_SCALE_PER_ROW;
+    const cudaError_t e = launch_pack_rows(geo, L->perm, W, N, per_row, Wp, s_w, s);
+    if (e != cudaErrorNotSupported) return cuda_status(e);
+    return cuda_status(launch_pack_weights(geo, L->perm, W, N, per_row, Wp, s_w, s));
 }
 
 int64_t soniq_quantize_act_scratch_bytes(const soniq_layout* L, int64_t M, int32_t scale_mode) {

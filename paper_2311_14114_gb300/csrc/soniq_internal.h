@@ -114,6 +114,11 @@ cudaError_t launch_pack_weights(const LayoutGeom& geo, const int32_t* perm, cons
                                 int32_t N, int32_t per_row, uint8_t* Wp, float* s_w,
                                 cudaStream_t st);
 
+// The same with bulk-staged rows (pack_rows.cu), for rows whose codes fit the
+// register tiles of one CTA (about 17,000 codes); cudaErrorNotSupported otherwise.
+cudaError_t launch_pack_rows(const LayoutGeom& geo, const int32_t* perm, const float* W, int32_t N, int32_t per_row,
+                             uint8_t* Wp, float* s_w, cudaStream_t st);
+
 // Layout variants (variant.cu): scales per (row or tensor, group, run), then
 // codes and packing; weights always per row.
 cudaError_t launch_variant_quantize_act(const LayoutGeom& geo, const int32_t* perm, const uint16_t* A, int64_t M,
