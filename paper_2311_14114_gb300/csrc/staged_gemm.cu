@@ -29,22 +29,26 @@
 //     over its K range could exceed that is accumulated in segments that the
 //     epilogue warps drain into int32 registers.
 //
-// The GEMM kernel: persistent CTAs (one per SM) walk 128 x 256 output tiles
-// (N = 256 per MMA: with 128-column MMAs the per-instruction cost, not the
-// tensor pipe, set the pace).
+// The GEMM kernel: persistent CTAs (one per SM) walk output tiles of 128 rows by
+// 256 columns (240, 128 or 64 where that fits the layout or the shape better;
+// pairs of CTAs: 256 x 256, or 240).
 //   warp 0      TMA producer: per 128-byte K-stage, an A box (128 rows, 16 KB)
-//               and a B box (256 rows, 32 KB), 128-byte swizzle, 4-stage ring
-//   warp 1      TMEM owner and MMA issuer (one thread): 4 MMAs per K-stage.
-//               A tile's accumulation is a sequence of jobs (a group, or one
-//               exact segment of a group; the segmented group first), and job
+//               and a B box, 128-byte swizzle, a ring as deep as shared memory allows
+//   warp 1      TMEM owner and MMA issuer: 4 MMAs per K-stage.
+//               A tile's accumulation is a sequence of jobs (a group, one
+//               exact segment of a group, or one scale run; the segmented group first), and job
 //               k of the CTA accumulates into TMEM region k % 2 (256 columns
 //               each), so the epilogue drains one region while the MMAs fill
 //               the other, across tile boundaries too
-//   warps 2-9   epilogue: two warps per TMEM lane quadrant, 128 columns each;
-//               earlier jobs of a tile are summed into int32 registers, the
-//               final job completes the outputs, which leave through shared
-//               memory and TMA stores (ten warps in all, so that each thread
-//               can hold 128 partial sums in registers)
+//   warps 4-11  epilogue: two warps per TMEM lane quadrant, half of the tile's
+//               columns each; earlier jobs of a tile are kept in registers,
+//               the final job completes the outputs
+// The issuing warps run their loops with all lanes and put only the TMA and MMA
+// instructions under an elected lane, so that descriptors and addresses stay in
+// uniform registers: under `lane == 0` each 4-MMA stage took 600-640 cycles to
+// issue, whatever the tile's width, where the pair's MMAs take 512 (the
+// 8192 x 4096 x 4096 4/8-bit call went from 121 to 109 us with this alone; its
+// MMAs without loads or epilogue take 75 us, and the operand expansion 22).
 // Every wait is bounded (2 s); a wait that runs out records an error bit,
 // raises a CTA abort flag and the CTA winds down (copies and MMAs in flight
 // are waited for, TMEM is freed).
@@ -68,34 +72,54 @@ constexpr int BN_F4 = 240;                           // tile width of layouts wi
 constexpr int REGION = 256;                          // TMEM columns per accumulator region
 constexpr int SF_COLS = 16;                          // E2M1 scale factors: region columns BN_F4 .. +15
 constexpr int KSTAGE = 128;                          // bytes of K per ring stage (128-byte swizzle)
-constexpr int STAGES = 3;
 constexpr int A_BYTES = BM * KSTAGE;
-constexpr int B_BYTES = BN * KSTAGE;
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int NUM_EPI_WARPS = 8;
-constexpr int WARP_TMA = 0, WARP_MMA = 1, WARP_EPI = 2;
-constexpr int NUM_THREADS = (2 + NUM_EPI_WARPS) * 32;
-constexpr int BAR_FULL = 0, BAR_EMPTY = STAGES, BAR_REG_FULL = 2 * STAGES, BAR_REG_EMPTY = 2 * STAGES + 2,
-              BAR_TEARDOWN = 2 * STAGES + 4, NUM_BARS = 2 * STAGES + 5;
-constexpr int EPI_COLS = BN / (NUM_EPI_WARPS / 4);     // columns per epilogue warp (128)
-constexpr int COLS_PER_WARP = EPI_COLS * 16;            // float4 per column: s_w0', s_w1', center*C0, center*C1
-constexpr int OUT_PER_WARP = 32 * EPI_COLS * 2;         // a warp's 32 x 128 outputs: two 64-column boxes, 128-byte swizzled
-constexpr int SMEM_OUT = STAGES * STAGE_BYTES;
-constexpr int SMEM_COLS = SMEM_OUT + NUM_EPI_WARPS * OUT_PER_WARP;
-constexpr int SMEM_BAR = SMEM_COLS + NUM_EPI_WARPS * COLS_PER_WARP;
-constexpr int SMEM_MISC = SMEM_BAR + NUM_BARS * 8;   // tmem base, abort flag, a zero word
-constexpr int SMEM_TOTAL = SMEM_MISC + 16;
-constexpr int SMEM_ALLOC = SMEM_TOTAL + 1024;        // slack for 1024-byte alignment
-constexpr int PAIR_STAGES = 4;                       // ring of the 2-SM kernel (32 KB stages)
+constexpr int WARP_TMA = 0, WARP_MMA = 1, WARP_EPI = 4;      // warps 2 and 3 only give up registers
+constexpr int NUM_THREADS = (WARP_EPI + NUM_EPI_WARPS) * 32;
 
-// Dynamic shared memory of the 2-SM instantiations: the ring, the output
-// staging tile, the column constants, the barriers and misc words, the slack.
-constexpr int pair_smem_alloc() {
-    return PAIR_STAGES * (A_BYTES + BN / 2 * KSTAGE) + NUM_EPI_WARPS * OUT_PER_WARP + NUM_EPI_WARPS * COLS_PER_WARP +
-           (2 * PAIR_STAGES + 5) * 8 + 16 + 1024;
-}
-static_assert(pair_smem_alloc() <= 227 * 1024, "the 2-SM ring fits");
-constexpr uint32_t IDESC = idesc(BM, BN);
+// Epilogues.  LEAN, SEG, NEXT and RUNS read the accumulators as MMA fragments
+// (fragment epilogue below); GENERAL and GENERAL_NEXT, one row per lane, also
+// write debug accumulators.
+enum {
+    EPI_LEAN = 0,          // both groups accumulated in one piece each
+    EPI_SEG = 1,           // one group in exact segments, drained to int32
+    EPI_NEXT = 2,          // LEAN, plus the next layer's codes (quantize-in-epilogue)
+    EPI_RUNS = 3,          // scale runs along K
+    EPI_GENERAL = 4,
+    EPI_GENERAL_NEXT = 5
+};
+
+// How outputs leave: OUT_BATCH stages 32 rows x 32 columns per epilogue warp
+// (2 KB) at a time and copies them out with 16-byte stores, which leaves the
+// shared memory to the operand ring (six 32 KB stages for a pair); OUT_TMA
+// stages a warp's whole tile (8 KB) for TMA stores, the quicker epilogue where
+// few K-stages per tile leave it on the critical path.  GEMM calls, batch
+// against TMA: 8192 x 4096 x 4096 4/8 bits (40 K-stages, pairs) 121 and 125 us, its
+// 2/8-bit layout with E2M1 groups 97 and 108 us, 16384 x 768 x 3072 (9 K-stages)
+// 75 and 69 us.
+enum { OUT_BATCH = 0, OUT_TMA = 1, OUT_GENERAL = 2 };
+
+// Shared memory of a variant: the operand ring, the epilogue warps' output
+// staging, the tile's column constants (16 bytes per column, two tiles' worth;
+// GENERAL: one copy per warp), the barriers, misc words (tmem base, abort flag,
+// a zero word).
+template <int BNT, bool PAIR, int OUT>
+struct Cfg {
+    static constexpr int B_BYTES = (PAIR ? BNT / 2 : BNT) * KSTAGE;
+    static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
+    static constexpr int STAGES = (OUT == OUT_BATCH ? 192 : 144) * 1024 / STAGE_BYTES;
+    static constexpr int EPI_COLS = BNT / (NUM_EPI_WARPS / 4);
+    static constexpr int COLS_BYTES = EPI_COLS * 16;               // constants of one warp's columns
+    static constexpr int OUT_PER_WARP = OUT != OUT_BATCH ? (32 * EPI_COLS * 2 + 1023) / 1024 * 1024 : 2048;
+    static constexpr int BAR_FULL = 0, BAR_EMPTY = STAGES, BAR_REG_FULL = 2 * STAGES, BAR_REG_EMPTY = 2 * STAGES + 2,
+                         BAR_TEARDOWN = 2 * STAGES + 4, BAR_COLS = 2 * STAGES + 5, NUM_BARS = 2 * STAGES + 9;
+    static constexpr int SMEM_OUT = STAGES * STAGE_BYTES;
+    static constexpr int SMEM_COLS = SMEM_OUT + NUM_EPI_WARPS * OUT_PER_WARP;
+    static constexpr int SMEM_BAR = SMEM_COLS + 8 * COLS_BYTES;
+    static constexpr int SMEM_MISC = SMEM_BAR + NUM_BARS * 8;
+    static constexpr int SMEM_ALLOC = SMEM_MISC + 16 + 1024;      // slack for 1024-byte alignment
+    static_assert(SMEM_ALLOC <= 227 * 1024, "the ring and the epilogue's buffers fit");
+};
 constexpr long long kTimeoutNs = 2000000000LL;
 
 struct SGroup {
@@ -111,8 +135,7 @@ struct SGroup {
 
 struct SParams {
     CUtensorMap tma_a;     // expanded activations [rows][eb]
-    CUtensorMap tma_b;     // expanded weights [N][eb]
-    CUtensorMap tma_b2;    // the same, 128-row boxes (each CTA of a pair loads half the tile's rows)
+    CUtensorMap tma_b;     // expanded weights [N][eb] (each CTA of a pair loads half the tile's rows)
     CUtensorMap tma_y;     // outputs [M][N] (2-byte elements), 64 x 32 boxes, when y_tma
     const float* s_a;
     const float* s_w;
@@ -362,50 +385,18 @@ __device__ __forceinline__ void store_out8(const SParams& p, int64_t m, int nb, 
     }
 }
 
-__device__ __forceinline__ void store_out16(const SParams& p, int64_t m, int nb, const float (&y)[16]) {
-    const bool vec = nb + 16 <= p.N && (p.N & 7) == 0;
-    if (p.out_bf16) {
-        __nv_bfloat16* dst = reinterpret_cast<__nv_bfloat16*>(p.Y) + m * p.N;
-        if (vec) {
-#pragma unroll
-            for (int v8 = 0; v8 < 2; ++v8) {
-                uint32_t wv[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(y[v8 * 8 + 2 * e], y[v8 * 8 + 2 * e + 1]);
-                    wv[e] = *reinterpret_cast<uint32_t*>(&h2);
-                }
-                *reinterpret_cast<uint4*>(dst + nb + v8 * 8) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-        } else {
-            for (int j = 0; j < 16; ++j)
-                if (nb + j < p.N) dst[nb + j] = __float2bfloat16_rn(y[j]);
-        }
-    } else {
-        __half* dst = reinterpret_cast<__half*>(p.Y) + m * p.N;
-        if (vec) {
-#pragma unroll
-            for (int v8 = 0; v8 < 2; ++v8) {
-                uint32_t wv[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    __half2 h2 = __floats2half2_rn(y[v8 * 8 + 2 * e], y[v8 * 8 + 2 * e + 1]);
-                    wv[e] = *reinterpret_cast<uint32_t*>(&h2);
-                }
-                *reinterpret_cast<uint4*>(dst + nb + v8 * 8) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
-            }
-        } else {
-            for (int j = 0; j < 16; ++j)
-                if (nb + j < p.N) dst[nb + j] = __float2half_rn(y[j]);
-        }
-    }
-}
-
 // The tile's accumulation jobs, in order: the group that needs exact
 // segments (if any) first, then the other one; each segment is one job.
 // Job k of the CTA accumulates into TMEM region k % 2 (256 columns), so the
 // epilogue drains one region while the MMAs fill the other.
 __device__ __forceinline__ int first_group(const SParams& p) { return p.seg_group == 1 ? 1 : 0; }
+
+// Shared address of 8-column block c (0..3) of row r in a warp's 32 x 32 batch
+// of staged outputs: 64-byte rows, swizzled so that 8 rows of a block, and the
+// 4 blocks of 2 rows, lie on distinct banks.
+__device__ __forceinline__ uint32_t batch_addr(uint32_t out_s, int c, int r) {
+    return out_s + (uint32_t)r * 64u + ((((uint32_t)c) ^ (((uint32_t)r >> 1) & 3u)) << 4);
+}
 
 // Quantize-in-epilogue (Sec. 4.1, Conv2D + BatchNorm + Quantize fused): the
 // next layer's packed codes of this lane's row from the fp16 outputs in the
@@ -414,11 +405,12 @@ __device__ __forceinline__ int first_group(const SParams& p) { return p.seg_grou
 // positions, so each 32-column block is one packed block of its group (Sec. 3
 // step 2 with the next layer's calibrated scale).  Kept out of the unrolled
 // output loop, with run-time widths, so that the kernel's code stays small.
-__device__ __forceinline__ void next_layer_codes(const SParams& p, uint32_t out_s, int lane, int m, int nc0) {
+__device__ __noinline__ void next_layer_codes(const SParams& p, uint32_t out_s, int lane, int64_t m, int nc0) {
+    constexpr int COLS = 128;
     const QConst kn0 = make_qconst(__ldg(p.s_next), p.next_bits[0]);
     const QConst kn1 = make_qconst(__ldg(p.s_next + 1), p.next_bits[1]);
 #pragma unroll 1
-    for (int b = 0; b < EPI_COLS / 32; ++b) {
+    for (int b = 0; b < COLS / 32; ++b) {
         const int cb = nc0 + 32 * b;                       // first column of the block
         if (cb >= p.N) break;
         const int gn = cb >= p.next_pa0;
@@ -458,112 +450,556 @@ __device__ __forceinline__ void next_layer_codes(const SParams& p, uint32_t out_
             o[2 * i + 1] = u[4] | (u[5] << 8) | (u[6] << 16) | (u[7] << 24);
         }
         const int nb = gn ? p.next_bits[1] : p.next_bits[0];
-        store_block32_rt(nb, o, p.Ap_next + m * (int64_t)p.next_row_bytes + (gn ? p.next_off[1] : p.next_off[0]) +
+        store_block32_rt(nb, o, p.Ap_next + m * p.next_row_bytes + (gn ? p.next_off[1] : p.next_off[0]) +
                                     (jg >> 5) * 4 * nb);
     }
 }
 
-// Scale runs along K (epilogue warp, one tile): every job is one run b of one
-// group g, drained as its exact integer sum and added in fp32 with its own
-// scale, y += s_a(g, b) s_w(n, g, b) / (La Lw) * Acc(g, b); then the tile's
-// outputs.  `kw` is this warp's 128-float scratch for a run's column scales.
-// With debug accumulators, acc_dbg receives [2][nb][M][N].  Returns false
-// after a wait ran out.
-__device__ __noinline__ bool runs_tile(const SParams& p, uint32_t sbase, uint32_t bar0, uint32_t abort_flag,
-                                       uint32_t lane_base, uint32_t out_s, float* kw, int lane, int quad, int64_t m,
-                                       int64_t m0, int nc0, uint32_t& job) {
-    auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    float yr[EPI_COLS];
+// ---------------------------------------------------------------------------
+// Fragment epilogue
+// ---------------------------------------------------------------------------
+//
+// What bounds it: next to the MMAs' operand traffic, shared-memory bandwidth
+// and instruction issue.  With one accumulator row per lane (the GENERAL
+// epilogue) every lane reads every column's constants, 16 bytes per output
+// element from shared memory, and each output takes four int/float
+// conversions, which issue at a sixteenth of the fp32 rate.  Two changes:
+//   * the accumulators are read as MMA fragments (tcgen05.ld 16x256b): a lane
+//     holds columns 8 c + 2 (lane % 4) + {0, 1} of rows lane / 4 + {0, 8, 16,
+//     24}, so one pair of 16-byte constants serves eight outputs, and
+//     stmatrix writes the 8 x 8 blocks to the staging tile;
+//   * an accumulator of one exact piece is an integer below 2^24 held in
+//     fp32: v * 2^18 (or 4, or 1) is that integer, and adding the centring
+//     term (an integer with at most 24 significant bits, also exact) rounds
+//     once, to the very value the conversion of the int32 sum gives.
+// Only segmented groups, whose sums may pass 2^24, go through int32.
+
+struct FragTile {
+    uint32_t bar0, abort_flag;
+    uint32_t tmem;             // the warp's TMEM lane quadrant and first column of region 0
+    uint32_t out_s;            // staging tile (shared address)
+    float4* colc;              // column constants (shared memory)
+    int quad, lane;
+    int cgrp;                  // column half of the tile
+    int tile;                  // tiles of this CTA so far
+    int64_t m0;                // first row of the warp's 32
+    int nc0;                   // its first column
+};
+
+#define SONIQ_R8(r, o) \
+    "=r"(r[o]), "=r"(r[o + 1]), "=r"(r[o + 2]), "=r"(r[o + 3]), "=r"(r[o + 4]), "=r"(r[o + 5]), "=r"(r[o + 6]), "=r"(r[o + 7])
+#define SONIQ_RW8(r, o) \
+    "+r"(r[o]), "+r"(r[o + 1]), "+r"(r[o + 2]), "+r"(r[o + 3]), "+r"(r[o + 4]), "+r"(r[o + 5]), "+r"(r[o + 6]), "+r"(r[o + 7])
+
+// Issues the loads of NC 8-column blocks of the quadrant's lanes 0..15 (v[0 ..
+// 4 NC - 1]) and 16..31 (v[8 ..], 4 NC of them).  v[4 j + {0, 1}]: row lane / 4,
+// columns 8 j + 2 (lane % 4) + {0, 1}; v[4 j + {2, 3}]: row lane / 4 + 8.  The
+// values are there after tmem_frag_wait on the same registers.
+template <int NC>
+__device__ __forceinline__ void tmem_frag_issue(uint32_t taddr, uint32_t (&v)[16]) {
+    const uint32_t hi = taddr + (16u << 16);
+    if constexpr (NC == 2) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+            "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];"
+            : SONIQ_R8(v, 0), SONIQ_R8(v, 8)
+            : "r"(taddr), "r"(hi));
+    } else {
+        static_assert(NC == 1, "1 or 2 blocks");
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%8];\n\t"
+            "tcgen05.ld.sync.aligned.16x256b.x1.b32 {%4,%5,%6,%7}, [%9];"
+            : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11])
+            : "r"(taddr), "r"(hi));
+        v[4] = v[5] = v[6] = v[7] = v[12] = v[13] = v[14] = v[15] = 0u;
+    }
+}
+
+// Waits for this thread's TMEM loads; v's registers pass through, so that no use of them moves up.
+__device__ __forceinline__ void tmem_frag_wait(uint32_t (&v)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : SONIQ_RW8(v, 0), SONIQ_RW8(v, 8)::"memory");
+}
+
+// Calls f(block, values) for 8-column blocks C .. NCH - 1, whose first two are
+// in (or on their way to) cur; the next two load while these are processed.
+// f's values: {0, 1} row lane / 4, {2, 3} + 8, {4, 5} + 16, {6, 7} + 24.
+template <int C, int NCH, typename F>
+__device__ __forceinline__ void frag_step(uint32_t taddr, uint32_t (&cur)[16], F& f) {
+    constexpr int N = NCH - C >= 2 ? 2 : 1;
+    tmem_frag_wait(cur);
+    uint32_t nxt[16];
+    if constexpr (C + N < NCH) tmem_frag_issue<(NCH - C - N >= 2 ? 2 : 1)>(taddr + 8 * (C + N), nxt);
 #pragma unroll
-    for (int j = 0; j < EPI_COLS; ++j) yr[j] = 0.0f;
-    const bool dbg = p.acc_dbg != nullptr && m < p.M;
-    for (int g = 0; g < 2; ++g) {
-        const int nrun = p.g[g].stages > 0 ? p.g[g].n_seg : 0;
-        const float sc = p.g[g].acc_scale;
-#pragma unroll 1
-        for (int b = 0; b < nrun; ++b, ++job) {
-            const uint32_t r = job & 1u, use = job >> 1;
-            if (!__all_sync(0xffffffffu, wait_bounded(bar(BAR_REG_FULL + r), use & 1u, abort_flag, kTimeoutNs,
-                                                      p.err, kErrWait)))
-                return false;
-            tc_fence_after();
-            __syncwarp();
+    for (int j = 0; j < N; ++j) {
+        const uint32_t v[8] = {cur[4 * j], cur[4 * j + 1], cur[4 * j + 2], cur[4 * j + 3],
+                               cur[8 + 4 * j], cur[9 + 4 * j], cur[10 + 4 * j], cur[11 + 4 * j]};
+        f(C + j, v);
+    }
+    if constexpr (C + N < NCH) frag_step<C + N, NCH>(taddr, nxt, f);
+}
+
+template <int NCH, typename F>
+__device__ __forceinline__ void frag_blocks(uint32_t taddr, F&& f) {
+    uint32_t first[16];
+    tmem_frag_issue<(NCH >= 2 ? 2 : 1)>(taddr, first);
+    frag_step<0, NCH>(taddr, first, f);
+}
+
+// Two fp32 operations per instruction (each element rounded as its scalar
+// counterpart).  Products and sums are spelled as fused multiply-adds with
+// -0 and 1, which nothing can fuse further.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return fma2(a, b, make_float2(-0.0f, -0.0f)); }
+
+// Four 8 x 8 blocks of 16-bit values (rows 0..31 of the warp); lane l gives the address of row l.
+__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&w)[4]) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]),
+                 "r"(w[2]), "r"(w[3]));
+}
+
+__device__ __forceinline__ uint32_t pack_out(float lo, float hi, int bf16) {
+    if (bf16) {
+        __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);
+        return *reinterpret_cast<uint32_t*>(&h);
+    }
+    __half2 h = __floats2half2_rn(lo, hi);
+    return *reinterpret_cast<uint32_t*>(&h);
+}
+
+// The warp's staged batch, columns cb .. cb + 8 nc - 1 of its 32 rows, to Y:
+// 16-byte stores, 64 contiguous bytes per row, or 4- or 2-byte ones where the
+// row pitch (N) is not a multiple of 8.  (TMA stores would share the TMA unit
+// with the operand loads.)
+__device__ __forceinline__ void batch_out(const SParams& p, const FragTile& t, int cb, int nc) {
+    __syncwarp();
+    const int ncol = min(8 * nc, p.N - cb);
+    if ((p.N & 7) == 0) {
+        const int c = t.lane & 3;
+        uint4* dst = reinterpret_cast<uint4*>(static_cast<uint16_t*>(p.Y) + (t.m0 + (t.lane >> 2)) * p.N + cb + 8 * c);
+        const int64_t rows = p.M - t.m0 - (t.lane >> 2);
 #pragma unroll
-            for (int h = 0; h < EPI_COLS / 32; ++h) {
-                const int c = lane + 32 * h;
-                const int n = nc0 + c < p.N ? nc0 + c : p.N - 1;
-                kw[c] = __ldg(p.s_w + ((int64_t)n * 2 + g) * p.nb + b) * p.g[g].inv_levels;
-            }
-            __syncwarp();
-            const float sa = m < p.M ? __ldg(p.s_a + ((p.s_a_per_row ? m : 0) * 2 + g) * p.nb + b) : 0.0f;
-            const uint32_t taddr = lane_base + r * REGION;
-#pragma unroll
-            for (int cc = 0; cc < EPI_COLS / 8; ++cc) {
-                uint32_t v[8];
-                tmem_ld8(taddr + cc * 8, v);
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    const int j = cc * 8 + q;
-                    const int32_t x = __float2int_rn(__uint_as_float(v[q]) * sc);
-                    yr[j] = fmaf(sa * kw[j], (float)x, yr[j]);
-                    if (dbg && nc0 + j < p.N)
-                        p.acc_dbg[(((int64_t)g * p.nb + b) * p.M + m) * p.N + nc0 + j] = x;
-                }
-            }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(BAR_REG_EMPTY + r));
+        for (int i = 0; i < 4; ++i) {
+            uint4 v;
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+                         : "r"(batch_addr(t.out_s, c, (t.lane >> 2) + 8 * i)));
+            if (8 * c < ncol && 8 * i < rows) dst[(int64_t)i * p.N] = v;       // 8 rows: N 16-byte vectors
+        }
+    } else if ((p.N & 1) == 0) {
+        const int c = 2 * (t.lane & 15);
+        for (int r = t.lane >> 4; r < 32 && t.m0 + r < p.M; r += 2) {
+            uint32_t v;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(batch_addr(t.out_s, c >> 3, r) + 2u * (c & 7)));
+            if (c < ncol) *reinterpret_cast<uint32_t*>(static_cast<uint16_t*>(p.Y) + (t.m0 + r) * p.N + cb + c) = v;
+        }
+    } else {
+        const int c = t.lane;
+        for (int r = 0; r < 32 && t.m0 + r < p.M; ++r) {
+            uint16_t v;
+            asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(batch_addr(t.out_s, c >> 3, r) + 2u * (c & 7)));
+            if (c < ncol) static_cast<uint16_t*>(p.Y)[(t.m0 + r) * p.N + cb + c] = v;
         }
     }
-    // the tile's outputs, 8 columns at a time
-    if (p.y_tma) {
+    __syncwarp();      // read before the next batch is staged
+}
+
+// Shared address of row r of 8-column block c of a warp's whole staged tile:
+// 64-column boxes of 128-byte-swizzled rows (the TMA store map's layout).
+__device__ __forceinline__ uint32_t staging_addr(uint32_t out_s, int c, int r) {
+    return out_s + (uint32_t)(c >> 3) * 4096u + (uint32_t)r * 128u + ((((uint32_t)c & 7u) ^ ((uint32_t)r & 7u)) << 4);
+}
+
+// The warp's whole staged tile leaves by TMA stores; rows and columns beyond M
+// and N are clipped.
+template <int EPI_COLS>
+__device__ __forceinline__ void staged_out(const SParams& p, const FragTile& t) {
+    static_assert(EPI_COLS % 64 == 0, "whole boxes");
+    fence_proxy_async_shared();
+    __syncwarp();
+    if (t.lane == 0) {
+#pragma unroll
+        for (int bx = 0; bx < EPI_COLS / 64; ++bx)
+            tma_store_2d(&p.tma_y, t.nc0 + bx * 64, (int)t.m0, t.out_s + bx * 4096u);
+        bulk_commit();
+    }
+}
+
+// Low bytes of four words, in order.
+__device__ __forceinline__ uint32_t low_bytes(uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
+    return __byte_perm(__byte_perm(b0, b1, 0x0040), __byte_perm(b2, b3, 0x0040), 0x5410);
+}
+
+// Sec. 3 step 2 on a pair of fp16 outputs under a calibrated scale (Markstein
+// quotient, the top clip on the input, rounding by adding 1.5 * 2^23: the
+// codes are the low bytes of the results).
+__device__ __forceinline__ void next_codes2(uint32_t h2, const QConst& k, uint32_t& c0, uint32_t& c1) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h2));
+    const float x0 = fmin_keep_nan(f.x, k.s), x1 = fmin_keep_nan(f.y, k.s);
+    const float p0 = __fmul_rn(x0, k.r), p1 = __fmul_rn(x1, k.r);
+    const float q0 = __fmaf_rn(__fmaf_rn(-p0, k.s, x0), k.r, p0), q1 = __fmaf_rn(__fmaf_rn(-p1, k.s, x1), k.r, p1);
+    c0 = __float_as_uint(__fadd_rn(fmaxf(__fmul_rn(q0, k.levels), 0.0f), 12582912.0f));
+    c1 = __float_as_uint(__fadd_rn(fmaxf(__fmul_rn(q1, k.levels), 0.0f), 12582912.0f));
+}
+
+// The next layer's packed codes from the warp's code bytes: cw[4 j + i] holds,
+// for 16-column block j and rows 8 i + lane / 4, the bytes of columns
+// 16 j + 2 (lane % 4) + {0, 1} and 16 j + 8 + 2 (lane % 4) + {0, 1}.  They
+// pass through the staging tile (128 bytes per row, swizzled); lane l then
+// packs row l, one 32-column block of one group at a time.
+template <int EPI_COLS>
+__device__ __forceinline__ void next_pack(const SParams& p, const FragTile& t, const uint32_t (&cw)[EPI_COLS / 4]) {
+    static_assert(EPI_COLS == 128, "128-byte rows");
+#pragma unroll
+    for (int j = 0; j < EPI_COLS / 16; ++j) {
+        const uint32_t w[4] = {cw[4 * j], cw[4 * j + 1], cw[4 * j + 2], cw[4 * j + 3]};
+        stmatrix4(staging_addr(t.out_s, j, t.lane), w);
+    }
+    __syncwarp();
+    const int64_t m = t.m0 + t.lane;
+    if (m >= p.M) return;
+    uint8_t* dst = p.Ap_next + m * p.next_row_bytes;
+#pragma unroll 1
+    for (int b = 0; b < EPI_COLS / 32; ++b) {
+        const int cb = t.nc0 + 32 * b;                     // first column of the block
+        if (cb >= p.N) break;
+        const int gn = cb >= p.next_pa0;
+        const int jg = cb - (gn ? p.next_pa0 : 0);         // position within the group
+        uint32_t o[8];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            uint32_t w[4];
+            asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                         : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3])
+                         : "r"(staging_addr(t.out_s, 2 * b + i, t.lane))
+                         : "memory");
+            // word q: columns 2q, 2q + 1 of the first eight (low half) and of the second eight
+            o[4 * i] = __byte_perm(w[0], w[1], 0x5410);
+            o[4 * i + 1] = __byte_perm(w[2], w[3], 0x5410);
+            o[4 * i + 2] = __byte_perm(w[0], w[1], 0x7632);
+            o[4 * i + 3] = __byte_perm(w[2], w[3], 0x7632);
+        }
+        const int valid = (gn ? p.next_count[1] : p.next_count[0]) - jg;   // real channels in the block
+        if (valid < 32) {
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int v = valid - 4 * q;               // padding positions hold code 0
+                o[q] &= v >= 4 ? 0xFFFFFFFFu : (v <= 0 ? 0u : (1u << (8 * v)) - 1u);
+            }
+        }
+        const int nb = gn ? p.next_bits[1] : p.next_bits[0];
+        store_block32_n(nb, o, dst + (gn ? p.next_off[1] : p.next_off[0]) + (jg >> 5) * 4 * nb);
+    }
+}
+
+// How a layer's tiles end: group gl completes with the tile's last job; group
+// gf (the first job's, or an absent one) is in registers by then.
+template <int EPI>
+struct ColPlan {
+    int gA, nA, njobs;         // the first jobs' group, its jobs, all jobs of a tile
+    int gf, gl;
+    bool both, same;           // two groups; SEG: earlier segments are of group gl itself
+    float invf, invl, scf, scl;
+    int centf, centl;          // centring of group f / l (0: none)
+    float saf, sal;            // per-tensor activation scales (1: per row)
+    __device__ __forceinline__ explicit ColPlan(const SParams& p) {
+        gA = EPI == EPI_SEG ? first_group(p) : 0;      // in segments only group gA may be
+        const int gB = 1 - gA;
+        nA = p.g[gA].stages > 0 ? p.g[gA].n_seg : 0;
+        const int nB = p.g[gB].stages > 0 ? p.g[gB].n_seg : 0;
+        njobs = nA + nB;
+        gl = nB > 0 ? gB : gA;
+        gf = 1 - gl;
+        both = nA > 0 && nB > 0;
+        same = EPI == EPI_SEG && !both;
+        invf = p.g[gf].inv_levels;
+        invl = p.g[gl].inv_levels;
+        scf = p.g[gf].acc_scale;
+        scl = p.g[gl].acc_scale;
+        centf = both ? p.g[gf].center : 0;
+        centl = p.g[gl].center;
+        saf = p.s_a_per_row ? 1.0f : __ldg(p.s_a + gf);
+        sal = p.s_a_per_row ? 1.0f : __ldg(p.s_a + gl);
+    }
+};
+
+// A tile's column constants {scale f, scale l, centring f, centring l}
+// (per-tensor: s_a included), 32 bytes per column pair: {scale f x 2, scale l
+// x 2}, {centring f x 2, centring l x 2}.  The four warps of a column half
+// each prepare a quarter of them: the global loads are issued before the
+// previous tile's last job, the stores follow it, and the half's barrier (one
+// per buffer) says that all four have arrived.
+struct ColLoad {
+    float2 sw;
+    int cf, cl;
+    template <int EPI>
+    __device__ __forceinline__ void load(const SParams& p, const ColPlan<EPI>& cp, const FragTile& t, int epi_cols) {
+        const int c = t.quad * (epi_cols / 4) + t.lane;
+        const int n = t.nc0 + c < p.N ? t.nc0 + c : p.N - 1;
+        sw = __ldg(reinterpret_cast<const float2*>(p.s_w) + n);
+        cf = cp.centf ? __ldg(p.colsum + (int64_t)n * 2 + cp.gf) : 0;
+        cl = cp.centl ? __ldg(p.colsum + (int64_t)n * 2 + cp.gl) : 0;
+    }
+    // into the buffer of tile number t.tile
+    template <typename C, int EPI>
+    __device__ __forceinline__ void store(const ColPlan<EPI>& cp, const FragTile& t) {
+        const int buf = t.tile & 1;
+        if (t.lane < C::EPI_COLS / 4) {
+            const int c = t.quad * (C::EPI_COLS / 4) + t.lane;
+            float* d = reinterpret_cast<float*>(t.colc) + buf * (C::COLS_BYTES / 4) + (c >> 1) * 8 + (c & 1);
+            d[0] = __fmul_rn(cp.saf, (cp.gf ? sw.y : sw.x) * cp.invf);
+            d[2] = __fmul_rn(cp.sal, (cp.gl ? sw.y : sw.x) * cp.invl);
+            // int32 where the group's sum is one, else fp32 (exact)
+            const int f = cp.centf * cf, l = cp.centl * cl;
+            d[4] = EPI == EPI_SEG ? __int_as_float(f) : (float)f;
+            d[6] = cp.same ? __int_as_float(l) : (float)l;
+        }
+        __syncwarp();
+        if (t.lane == 0) mbar_arrive(t.bar0 + 8u * (uint32_t)(C::BAR_COLS + 2 * t.cgrp + buf));
+    }
+};
+
+// One tile of an epilogue warp: waits for the tile's jobs, drains them and
+// writes the outputs (NEXT: also the next layer's codes); prepares tile nxt's
+// column constants (nxt.nc0 < 0: there is none).  release(r) hands TMEM region
+// r back.  False after a wait ran out.
+template <int EPI, bool ROWS, int BNT, bool PAIR, int OUT, typename Release>
+__device__ __forceinline__ bool frag_tile(const SParams& p, const ColPlan<EPI>& cp, const FragTile& t, FragTile& nxt,
+                                          ColLoad& cl, uint32_t& job, Release&& release) {
+    using C = Cfg<BNT, PAIR, OUT>;
+    constexpr int EPI_COLS = C::EPI_COLS, NCH = EPI_COLS / 8;
+    constexpr bool SEG = EPI == EPI_SEG, NEXT = EPI == EPI_NEXT;
+    const int lane = t.lane;
+    auto wait = [&](int b, uint32_t ph) {
+        return __all_sync(0xffffffffu, wait_bounded(t.bar0 + 8u * (uint32_t)b, ph, t.abort_flag, kTimeoutNs, p.err,
+                                                    kErrWait)) != 0;
+    };
+    // activation scales of this lane's four rows, groups f and l
+    float2 saf[4], sal[4];
+    if constexpr (ROWS) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int64_t m = t.m0 + 8 * r + (lane >> 2);
+            float f = 1.0f, l = 1.0f;
+            if (p.s_a_per_row) {
+                f = m < p.M ? __ldg(p.s_a + m * 2 + cp.gf) : 0.0f;
+                l = m < p.M ? __ldg(p.s_a + m * 2 + cp.gl) : 0.0f;
+            }
+            saf[r] = make_float2(f, f);
+            sal[r] = make_float2(l, l);
+        }
+    }
+
+    // ---- earlier jobs: the whole first group, or segments ----
+    uint32_t part[NCH * 8];                          // accumulators as they are, or int32 sums (SEG)
+#pragma unroll
+    for (int i = 0; i < NCH * 8; ++i) part[i] = 0u;
+#pragma unroll 1
+    for (int jj = 0; jj < cp.njobs - 1; ++jj, ++job) {
+        const uint32_t r = job & 1u, use = job >> 1;
+        if (!wait(C::BAR_REG_FULL + (int)r, use & 1u)) return false;
+        tc_fence_after();
+        const float sc = p.g[jj < cp.nA ? cp.gA : 1 - cp.gA].acc_scale;
+        frag_blocks<NCH>(t.tmem + r * REGION, [&](int c, const uint32_t (&v)[8]) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                if constexpr (SEG) part[8 * c + e] += (uint32_t)__float2int_rn(__fmul_rn(__uint_as_float(v[e]), sc));
+                else part[8 * c + e] = v[e];
+            }
+        });
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) release(r);
+    }
+
+    // ---- the final job ----
+    if (nxt.nc0 >= 0) cl.load(p, cp, nxt, EPI_COLS);
+    const int buf = t.tile & 1;
+    if (!wait(C::BAR_COLS + 2 * t.cgrp + buf, (uint32_t)(t.tile >> 1) & 1u)) return false;
+    const uint32_t r = job & 1u, use = job >> 1;
+    ++job;
+    if (!wait(C::BAR_REG_FULL + (int)r, use & 1u)) return false;
+    tc_fence_after();
+    QConst kn0, kn1;
+    bool codes_here = false;
+    if constexpr (NEXT) {
+        kn0 = make_qconst(__ldg(p.s_next), p.next_bits[0]);
+        kn1 = make_qconst(__ldg(p.s_next + 1), p.next_bits[1]);
+        // scales outside the Markstein range: from the staged outputs, below
+        codes_here = kn0.mode == 1 && kn1.mode == 1;
+    }
+    const bool stage_y = !NEXT || p.write_y || !codes_here;
+    if constexpr (OUT == OUT_TMA) {
+        // the previous tile's store must have read the staging tile
         if (lane == 0) bulk_wait_read0();
         __syncwarp();
     }
+    const float4* kc = t.colc + buf * (C::COLS_BYTES / 16) + 2 * (lane & 3);
+    const float2 scf = make_float2(cp.scf, cp.scf), scl = make_float2(cp.scl, cp.scl);
+    uint32_t cw[NEXT ? EPI_COLS / 4 : 1];
+    uint32_t cprev[NEXT ? 8 : 1];
+    frag_blocks<NCH>(t.tmem + r * REGION, [&](int c, const uint32_t (&v)[8]) {
+        const float4 ks = kc[8 * c], ct = kc[8 * c + 1];     // scales, centrings of the lane's two columns
+        uint32_t w[4];
 #pragma unroll
-    for (int cc = 0; cc < EPI_COLS / 8; ++cc) {
-        float y[8];
-#pragma unroll
-        for (int q = 0; q < 8; ++q) y[q] = yr[cc * 8 + q];
-        if (p.y_tma) {
-            uint32_t w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (p.out_bf16) {
-                    __nv_bfloat162 h2 = __floats2bfloat162_rn(y[2 * e], y[2 * e + 1]);
-                    w[e] = *reinterpret_cast<uint32_t*>(&h2);
-                } else {
-                    __half2 h2 = __floats2half2_rn(y[2 * e], y[2 * e + 1]);
-                    w[e] = *reinterpret_cast<uint32_t*>(&h2);
-                }
+        for (int i = 0; i < 4; ++i) {                          // row lane / 4 + 8 i
+            float2 kf = make_float2(ks.x, ks.y), kl = make_float2(ks.z, ks.w);
+            if constexpr (ROWS) {
+                kf = mul2(saf[i], kf);
+                kl = mul2(sal[i], kl);
             }
-            const uint32_t dst = out_s + (uint32_t)(cc >> 3) * 4096u + (uint32_t)lane * 128u +
-                                 ((((uint32_t)cc & 7u) ^ ((uint32_t)lane & 7u)) << 4);
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(w[0]), "r"(w[1]), "r"(w[2]),
-                         "r"(w[3])
-                         : "memory");
-        } else if (m < p.M) {
-            store_out8(p, m, nc0 + cc * 8, y);
+            const float2 vl = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+            const uint32_t p0 = part[8 * c + 2 * i], p1 = part[8 * c + 2 * i + 1];
+            float2 y;
+            if constexpr (SEG) {
+                float2 xl, xf;
+                if (cp.same) {
+                    const int x0 = (int)p0 + __float2int_rn(__fmul_rn(vl.x, cp.scl)) + __float_as_int(ct.z);
+                    const int x1 = (int)p1 + __float2int_rn(__fmul_rn(vl.y, cp.scl)) + __float_as_int(ct.w);
+                    xl = make_float2((float)x0, (float)x1);
+                    xf = make_float2(0.0f, 0.0f);
+                } else {
+                    xl = fma2(vl, scl, make_float2(ct.z, ct.w));
+                    xf = make_float2((float)((int)p0 + __float_as_int(ct.x)), (float)((int)p1 + __float_as_int(ct.y)));
+                }
+                // group 0's product is rounded first
+                y = cp.gf == 0 ? fma2(kl, xl, mul2(kf, xf)) : fma2(kf, xf, mul2(kl, xl));
+            } else {
+                const float2 vf = make_float2(__uint_as_float(p0), __uint_as_float(p1));
+                const float2 xl = fma2(vl, scl, make_float2(ct.z, ct.w));
+                const float2 xf = fma2(vf, scf, make_float2(ct.x, ct.y));
+                y = fma2(kl, xl, mul2(kf, xf));
+            }
+            w[i] = pack_out(y.x, y.y, NEXT ? 0 : p.out_bf16);
         }
-    }
-    if (p.y_tma) {
-        fence_proxy_async_shared();
-        __syncwarp();
-        if (lane == 0) {
+        if (stage_y) stmatrix4(OUT == OUT_BATCH ? batch_addr(t.out_s, c & 3, lane) : staging_addr(t.out_s, c, lane), w);
+        if constexpr (NEXT) {
+            // a 32-column block has one group, so this test is warp-uniform
+            const bool g1 = t.nc0 + 8 * c >= p.next_pa0;
+            QConst k;
+            k.s = g1 ? kn1.s : kn0.s;
+            k.r = g1 ? kn1.r : kn0.r;
+            k.levels = g1 ? kn1.levels : kn0.levels;
 #pragma unroll
-            for (int bx = 0; bx < EPI_COLS / 64; ++bx)
-                tma_store_2d(&p.tma_y, nc0 + bx * 64, (int)(m0 + quad * 32), out_s + bx * 4096u);
-            bulk_commit();
+            for (int i = 0; i < 4; ++i) {
+                uint32_t c0, c1;
+                next_codes2(w[i], k, c0, c1);
+                if (c & 1) cw[4 * (c >> 1) + i] = low_bytes(cprev[2 * i], cprev[2 * i + 1], c0, c1);
+                cprev[2 * i] = c0;
+                cprev[2 * i + 1] = c1;
+            }
         }
+        if constexpr (OUT == OUT_BATCH)
+            if ((c & 3) == 3 || c == NCH - 1) batch_out(p, t, t.nc0 + 32 * (c >> 2), (c & 3) + 1);
+    });
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) release(r);
+    if constexpr (OUT == OUT_TMA)
+        if (!NEXT || p.write_y) staged_out<EPI_COLS>(p, t);
+    if (nxt.nc0 >= 0) {
+        nxt.tile = t.tile + 1;
+        cl.store<C>(cp, nxt);
+    }
+    if constexpr (NEXT) {
+        if (codes_here) {
+            if (p.write_y) {
+                if (lane == 0) bulk_wait_read0();    // the outputs' store has read the staging tile
+                __syncwarp();
+            }
+            next_pack<EPI_COLS>(p, t, cw);
+        } else {
+            __syncwarp();
+            if (t.m0 + lane < p.M) next_layer_codes(p, t.out_s, lane, t.m0 + lane, t.nc0);
+        }
+        __syncwarp();
     }
     return true;
 }
 
-// Instantiations: GENERAL = false compiles the common epilogue lean (no debug
-// accumulators, outputs through TMA stores), which keeps the unrolled output
-// loop small enough for the instruction cache; GENERAL = true handles the
-// rest.  NEXT adds the next layer's codes (quantize-in-epilogue).
-template <bool GENERAL, bool NEXT, int BNT, bool PAIR>
+// Scale runs along K, one tile of an epilogue warp: every job is one run b of
+// one group g, whose exact integer sum is added in fp32 with its own scale,
+// y += (s_a(g, b) s_w(n, g, b) / (La Lw)) * Acc(g, b).  A job's scales are
+// loaded while the previous job is drained.  With debug accumulators, acc_dbg
+// receives [2][nb][M][N].  False after a wait ran out.
+template <int BNT, bool PAIR, typename Release>
+__device__ __forceinline__ bool runs_tile(const SParams& p, const FragTile& t, uint32_t& job, Release&& release) {
+    using C = Cfg<BNT, PAIR, OUT_BATCH>;
+    constexpr int EPI_COLS = C::EPI_COLS, NCH = EPI_COLS / 8, NK = EPI_COLS / 32;
+    const int lane = t.lane;
+    const int n0 = p.g[0].stages > 0 ? p.g[0].n_seg : 0, n1 = p.g[1].stages > 0 ? p.g[1].n_seg : 0;
+    float* kcol = reinterpret_cast<float*>(t.colc);
+    // scales of run jj: of the columns lane + 32 h, and of this lane's rows
+    float kw[NK], sa[4];
+    auto load_scales = [&](int jj) {
+        const int g = jj < n0 ? 0 : 1, b = g ? jj - n0 : jj;
+#pragma unroll
+        for (int h = 0; h < NK; ++h) {
+            const int n = t.nc0 + lane + 32 * h < p.N ? t.nc0 + lane + 32 * h : p.N - 1;
+            kw[h] = __ldg(p.s_w + ((int64_t)n * 2 + g) * p.nb + b);
+        }
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            const int64_t m = t.m0 + 8 * r + (lane >> 2);
+            sa[r] = m < p.M ? __ldg(p.s_a + ((p.s_a_per_row ? m : 0) * 2 + g) * p.nb + b) : 0.0f;
+        }
+    };
+    float y[NCH * 8];
+#pragma unroll
+    for (int i = 0; i < NCH * 8; ++i) y[i] = 0.0f;
+    if (n0 + n1 > 0) load_scales(0);
+#pragma unroll 1
+    for (int jj = 0; jj < n0 + n1; ++jj, ++job) {
+        const int g = jj < n0 ? 0 : 1, b = g ? jj - n0 : jj;
+        const float sc = p.g[g].acc_scale, inv = p.g[g].inv_levels;
+        __syncwarp();
+#pragma unroll
+        for (int h = 0; h < NK; ++h)
+            kcol[lane + 32 * h] = __fmul_rn(kw[h], inv);
+        __syncwarp();
+        const float s[4] = {sa[0], sa[1], sa[2], sa[3]};
+        if (jj + 1 < n0 + n1) load_scales(jj + 1);
+        const uint32_t r = job & 1u, use = job >> 1;
+        if (!__all_sync(0xffffffffu, wait_bounded(t.bar0 + 8u * (C::BAR_REG_FULL + r), use & 1u, t.abort_flag,
+                                                  kTimeoutNs, p.err, kErrWait)))
+            return false;
+        tc_fence_after();
+        frag_blocks<NCH>(t.tmem + r * REGION, [&](int c, const uint32_t (&v)[8]) {
+            const float2 kk = *reinterpret_cast<const float2*>(kcol + 8 * c + 2 * (lane & 3));
+            const float k[2] = {kk.x, kk.y};
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float x = __fmul_rn(__uint_as_float(v[e]), sc);       // the exact integer sum
+                y[8 * c + e] = __fmaf_rn(__fmul_rn(s[e >> 1], k[e & 1]), x, y[8 * c + e]);
+                if (p.acc_dbg != nullptr) {
+                    const int64_t m = t.m0 + 8 * (e >> 1) + (lane >> 2);
+                    const int n = t.nc0 + 8 * c + 2 * (lane & 3) + (e & 1);
+                    if (m < p.M && n < p.N) p.acc_dbg[(((int64_t)g * p.nb + b) * p.M + m) * p.N + n] = __float2int_rn(x);
+                }
+            }
+        });
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) release(r);
+    }
+#pragma unroll
+    for (int c = 0; c < NCH; ++c) {
+        uint32_t w[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = pack_out(y[8 * c + 2 * i], y[8 * c + 2 * i + 1], p.out_bf16);
+        stmatrix4(batch_addr(t.out_s, c & 3, lane), w);
+        if ((c & 3) == 3) batch_out(p, t, t.nc0 + 32 * (c >> 2), 4);
+    }
+    return true;
+}
+
+template <int EPI, bool ROWS, int BNT, bool PAIR, int OUT>
 __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid_constant__ SParams p) {
     // the tile width and what follows from it (BNT = 240: layouts with E2M1 groups,
     // whose block scale factors sit in the 16 TMEM columns past each region's tile)
@@ -575,22 +1011,21 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
     // commits arrive on both CTAs' empty and region-full barriers; both CTAs'
     // epilogue warps arrive on its region-empty barriers.
     static_assert(!PAIR || (BNT / 2) % 8 == 0, "pairs split B boxes into halves of whole 8-row swizzle atoms");
+    using C = Cfg<BNT, PAIR, OUT>;
     constexpr int BN = BNT;
-    constexpr int B_BYTES = (PAIR ? BN / 2 : BN) * KSTAGE;
-    constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-    constexpr int EPI_COLS = BN / (NUM_EPI_WARPS / 4);
-    constexpr int STAGES = PAIR ? PAIR_STAGES : staged::STAGES;
-    constexpr int BAR_FULL = 0, BAR_EMPTY = STAGES, BAR_REG_FULL = 2 * STAGES, BAR_REG_EMPTY = 2 * STAGES + 2,
-                  BAR_TEARDOWN = 2 * STAGES + 4, NUM_BARS = 2 * STAGES + 5;
+    constexpr int STAGE_BYTES = C::STAGE_BYTES, STAGES = C::STAGES, EPI_COLS = C::EPI_COLS;
+    constexpr int COLS_BYTES = C::COLS_BYTES, OUT_PER_WARP = C::OUT_PER_WARP;
+    static_assert((EPI >= EPI_GENERAL) == (OUT == OUT_GENERAL) && (EPI != EPI_NEXT || OUT == OUT_TMA), "epilogue and outputs");
+    constexpr int BAR_FULL = C::BAR_FULL, BAR_EMPTY = C::BAR_EMPTY, BAR_REG_FULL = C::BAR_REG_FULL,
+                  BAR_REG_EMPTY = C::BAR_REG_EMPTY, BAR_TEARDOWN = C::BAR_TEARDOWN;
+    constexpr int SMEM_OUT = C::SMEM_OUT, SMEM_COLS = C::SMEM_COLS, SMEM_BAR = C::SMEM_BAR, SMEM_MISC = C::SMEM_MISC;
+    constexpr bool GENERAL = EPI == EPI_GENERAL || EPI == EPI_GENERAL_NEXT;
+    constexpr bool F4 = BNT == BN_F4;    // layouts with E2M1 groups
     constexpr uint32_t IDESC2 = idesc(2 * BM, BN);
     constexpr uint32_t IDESC2_F4 = idesc_mxf4(2 * BM, BN);
-    constexpr int SMEM_OUT = STAGES * STAGE_BYTES;
-    constexpr int SMEM_COLS = SMEM_OUT + NUM_EPI_WARPS * OUT_PER_WARP;
-    constexpr int SMEM_BAR = SMEM_COLS + NUM_EPI_WARPS * COLS_PER_WARP;
-    constexpr int SMEM_MISC = SMEM_BAR + NUM_BARS * 8;
     constexpr uint32_t IDESC = idesc(BM, BN);
     constexpr uint32_t IDESC_F4 = idesc_mxf4(BM, BN);
-    constexpr bool BOX8 = BN != 256;     // outputs leave in 8-column boxes (EPI_COLS is not a multiple of 64)
+    constexpr bool BOX8 = EPI_COLS % 64 != 0;     // outputs leave in 8-column boxes
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -629,6 +1064,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
             mbar_init(bar(BAR_REG_EMPTY + i), PAIR ? 2 * NUM_EPI_WARPS : NUM_EPI_WARPS);
         }
         mbar_init(bar(BAR_TEARDOWN), 1);
+        for (int i = 0; i < 4; ++i) mbar_init(bar(C::BAR_COLS + i), NUM_EPI_WARPS / 2);
         set_flag(abort_flag, 0);
         set_flag(no_abort, 0);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -653,7 +1089,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot;
-    if constexpr (BN != REGION) {
+    if constexpr (F4) {
         // the E2M1 block scale factors: UE8M0 2^0 in every byte of each region's
         // spare columns (one epilogue warp per TMEM lane quadrant)
         if (warp >= WARP_EPI && warp < WARP_EPI + 4) {
@@ -672,10 +1108,15 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
     // written before this (the prologue above touches no global memory)
     pdl_wait();
 
-    if (warp == WARP_TMA) {
-        // ------------------------------------------------------------ producer
-        if (lane == 0) {
-            uint32_t s = 0;
+    // The launch gives every thread 168 registers; the epilogue's 128 partial
+    // sums and loads in flight need more (168 spilled 40 of them), so the first
+    // warpgroup hands its share over: 128 x 40 + 256 x 232 = 384 x 168.
+    if (warp < WARP_EPI) {
+        asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+        if (warp == WARP_TMA) {
+            // -------------------------------------------------------- producer
+            const bool leader = elect_one();
+            uint32_t s = 0, slot = 0, ph = 0;
             bool ok = true;
             for (int u = first_u; u < n_units && ok; u += step_u) {
                 const int m0 = tile_m(u) * BM, n0 = tile_n(u) * BN;
@@ -685,24 +1126,33 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                     const int ns = p.g[g].stages, x0 = p.g[g].x0;
 #pragma unroll 1
                     for (int i = 0; i < ns; ++i, ++s) {
-                        const uint32_t slot = s % STAGES, ph = (s / STAGES) & 1u;
-                        if (!wait_bounded(bar(BAR_EMPTY + slot), ph ^ 1u, abort_flag, kTimeoutNs, p.err, kErrWait)) {
+                        if (!wait_bounded_warp(bar(BAR_EMPTY + slot), ph ^ 1u, abort_flag, kTimeoutNs, p.err,
+                                               kErrWait)) {
                             ok = false;
                             break;
                         }
-                        if (p.drop_first && s == 0) continue;   // the MMA's wait for it runs out
                         const uint32_t dst = sbase + slot * STAGE_BYTES;
-                        if constexpr (PAIR) {
-                            // this CTA's A rows and B half; both CTAs' bytes complete on the
-                            // issuing CTA's full barrier
-                            const uint32_t fb = mapa_shared(bar(BAR_FULL + slot), 0u);
-                            if (issuer) mbar_arrive_expect_tx(bar(BAR_FULL + slot), 2 * STAGE_BYTES);
-                            tma_load_2d_pair(dst, &p.tma_a, x0 + i * KSTAGE, m0, fb);
-                            tma_load_2d_pair(dst + A_BYTES, &p.tma_b2, x0 + i * KSTAGE, n0 + (int)rank * (BN / 2), fb);
-                        } else {
-                            mbar_arrive_expect_tx(bar(BAR_FULL + slot), STAGE_BYTES);
-                            tma_load_2d(dst, &p.tma_a, x0 + i * KSTAGE, m0, bar(BAR_FULL + slot));
-                            tma_load_2d(dst + A_BYTES, &p.tma_b, x0 + i * KSTAGE, n0, bar(BAR_FULL + slot));
+                        if (p.drop_first && s == 0) {
+                            // the MMA's wait for this stage runs out
+                        } else if (leader) {
+                            if constexpr (PAIR) {
+                                // this CTA's A rows and B half; both CTAs' bytes complete on the
+                                // issuing CTA's full barrier
+                                const uint32_t fb = mapa_shared(bar(BAR_FULL + slot), 0u);
+                                if (issuer) mbar_arrive_expect_tx(bar(BAR_FULL + slot), 2 * STAGE_BYTES);
+                                tma_load_2d_pair(dst, &p.tma_a, x0 + i * KSTAGE, m0, fb);
+                                tma_load_2d_pair(dst + A_BYTES, &p.tma_b, x0 + i * KSTAGE, n0 + (int)rank * (BN / 2),
+                                                 fb);
+                            } else {
+                                mbar_arrive_expect_tx(bar(BAR_FULL + slot), STAGE_BYTES);
+                                tma_load_2d(dst, &p.tma_a, x0 + i * KSTAGE, m0, bar(BAR_FULL + slot));
+                                tma_load_2d(dst + A_BYTES, &p.tma_b, x0 + i * KSTAGE, n0, bar(BAR_FULL + slot));
+                            }
+                        }
+                        __syncwarp();
+                        if (++slot == (uint32_t)STAGES) {
+                            slot = 0;
+                            ph ^= 1u;
                         }
                     }
                 }
@@ -715,13 +1165,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                     if (!(p.drop_first && q == 0))
                         wait_bounded(bar(BAR_FULL + q % STAGES), (q / STAGES) & 1u, no_abort, kTimeoutNs, p.err,
                                      kErrWait);
-        }
-    } else if (warp == WARP_MMA) {
-        // ------------------------------------------------------------------ MMA
-        if (lane == 0 && issuer) {
-            uint32_t s = 0, job = 0;
+        } else if (warp == WARP_MMA && issuer) {
+            // -------------------------------------------------------------- MMA
+            const bool leader = elect_one();
+            uint32_t slot = 0, ph = 0, job = 0;
             bool ok = true;
-            const uint64_t a_desc0 = KSTAGE == 128 ? sw128_desc(sbase) : sw64_desc(sbase);
+            const uint64_t a_desc0 = sw128_desc(sbase);
             for (int u = first_u; u < n_units && ok; u += step_u) {
 #pragma unroll 1
                 for (int gi = 0; gi < 2 && ok; ++gi) {
@@ -732,8 +1181,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
 #pragma unroll 1
                     for (int i = 0; i < ns && ok; ++job) {
                         const uint32_t r = job & 1u, use = job >> 1;
-                        if (!wait_bounded(bar(BAR_REG_EMPTY + r), (use & 1u) ^ 1u, abort_flag, kTimeoutNs, p.err,
-                                          kErrWait)) {
+                        if (!wait_bounded_warp(bar(BAR_REG_EMPTY + r), (use & 1u) ^ 1u, abort_flag, kTimeoutNs, p.err,
+                                               kErrWait)) {
                             ok = false;
                             break;
                         }
@@ -741,9 +1190,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                         const uint32_t d = tmem_base + r * REGION;
                         const int jn = per_job < ns - i ? per_job : ns - i;
 #pragma unroll 1
-                        for (int q = 0; q < jn; ++q, ++i, ++s) {
-                            const uint32_t slot = s % STAGES, ph = (s / STAGES) & 1u;
-                            if (!wait_bounded(bar(BAR_FULL + slot), ph, abort_flag, kTimeoutNs, p.err, kErrWait)) {
+                        for (int q = 0; q < jn; ++q, ++i) {
+                            if (!wait_bounded_warp(bar(BAR_FULL + slot), ph, abort_flag, kTimeoutNs, p.err, kErrWait)) {
                                 ok = false;
                                 break;
                             }
@@ -751,41 +1199,42 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                             // descriptors of this stage; +32 bytes of K is +2 in the start-address field
                             const uint64_t ad = a_desc0 + (uint64_t)((slot * STAGE_BYTES) >> 4);
                             const uint64_t bd = ad + (uint64_t)(A_BYTES >> 4);
-                            if (PAIR && f4) {
-                                // unit block scales in the spare columns of this region in both CTAs
-                                const uint32_t sf = d + (uint32_t)BN_F4;
+                            const uint32_t sf = d + (uint32_t)BN_F4;   // E2M1: this region's unit block scales
+                            if (leader) {
+                                // (one unrolled run of MMAs per operand kind: the kind's branch
+                                // inside the run cost the headline call 12 us)
+                                auto run = [&](auto&& mma) {
 #pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma2_f4(d, ad + 2 * k, bd + 2 * k, IDESC2_F4, sf, sf + 8u, (q == 0 && k == 0) ? 0u : 1u);
-                            } else if (PAIR && f8) {
-#pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma2_f8<IDESC2>(d, ad + 2 * k, bd + 2 * k, (q == 0 && k == 0) ? 0u : 1u);
-                            } else if (PAIR) {
-#pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma2_f16<IDESC2>(d, ad + 2 * k, bd + 2 * k, (q == 0 && k == 0) ? 0u : 1u);
-                            } else if (f8) {
-#pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma_f8<IDESC>(d, ad + 2 * k, bd + 2 * k, (q == 0 && k == 0) ? 0u : 1u);
-                            } else if (f4) {
-                                // unit block scales (UE8M0 0x7F = 2^0) in this region's spare columns
-                                const uint32_t sf = d + (uint32_t)BN_F4;
-#pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma_f4(d, ad + 2 * k, bd + 2 * k, IDESC_F4, sf, sf + 8u,
-                                           (q == 0 && k == 0) ? 0u : 1u);
-                            } else {
-#pragma unroll
-                                for (int k = 0; k < KSTAGE / 32; ++k)
-                                    mma_f16<IDESC>(d, ad + 2 * k, bd + 2 * k, (q == 0 && k == 0) ? 0u : 1u);
+                                    for (int k = 0; k < KSTAGE / 32; ++k)
+                                        mma(ad + 2 * k, bd + 2 * k, (q == 0 && k == 0) ? 0u : 1u);
+                                };
+                                if (F4 && f4) {
+                                    run([&](uint64_t x, uint64_t y, uint32_t acc) {
+                                        if constexpr (PAIR) mma2_f4(d, x, y, IDESC2_F4, sf, sf + 8u, acc);
+                                        else mma_f4(d, x, y, IDESC_F4, sf, sf + 8u, acc);
+                                    });
+                                } else if (f8) {
+                                    run([&](uint64_t x, uint64_t y, uint32_t acc) {
+                                        if constexpr (PAIR) mma2_f8<IDESC2>(d, x, y, acc);
+                                        else mma_f8<IDESC>(d, x, y, acc);
+                                    });
+                                } else {
+                                    run([&](uint64_t x, uint64_t y, uint32_t acc) {
+                                        if constexpr (PAIR) mma2_f16<IDESC2>(d, x, y, acc);
+                                        else mma_f16<IDESC>(d, x, y, acc);
+                                    });
+                                }
+                                // the stage's slot is free again (in both CTAs)
+                                if constexpr (PAIR) mma2_commit_mc(bar(BAR_EMPTY + slot), (uint16_t)0x3);
+                                else mma_commit(bar(BAR_EMPTY + slot));
                             }
-                            // the stage's slot is free again in both CTAs
-                            if constexpr (PAIR) mma2_commit_mc(bar(BAR_EMPTY + slot), (uint16_t)0x3);
-                            else mma_commit(bar(BAR_EMPTY + slot));
+                            __syncwarp();
+                            if (++slot == (uint32_t)STAGES) {
+                                slot = 0;
+                                ph ^= 1u;
+                            }
                         }
-                        if (ok) {
+                        if (ok && leader) {
                             if constexpr (PAIR) mma2_commit_mc(bar(BAR_REG_FULL + r), (uint16_t)0x3);
                             else mma_commit(bar(BAR_REG_FULL + r));
                         }
@@ -793,12 +1242,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                 }
             }
             // every issued MMA completes before TMEM and shared memory are released
-            if constexpr (PAIR) mma2_commit(bar(BAR_TEARDOWN));
-            else mma_commit(bar(BAR_TEARDOWN));
+            if (leader) {
+                if constexpr (PAIR) mma2_commit(bar(BAR_TEARDOWN));
+                else mma_commit(bar(BAR_TEARDOWN));
+            }
+            __syncwarp();
             wait_bounded(bar(BAR_TEARDOWN), 0u, no_abort, kTimeoutNs, p.err, kErrWait);
         }
     } else {
         // ------------------------------------------------------------- epilogue
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
         // Warp w reads TMEM lane quadrant w % 4 (rows 32*(w%4) .. +31 of the
         // tile) and the 128 columns cgrp*128 .. +127, cgrp = (w - 2) / 4.
         const int ew = warp - WARP_EPI;
@@ -808,7 +1261,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(cgrp * EPI_COLS);
         // this warp's copy of the tile's column constants: {s_w0 * inv_levels0,
         // s_w1 * inv_levels1, center0 * C0, center1 * C1} per column
-        float4* colc = reinterpret_cast<float4*>(smem + SMEM_COLS + ew * COLS_PER_WARP);
+        float4* colc = reinterpret_cast<float4*>(smem + SMEM_COLS + ew * COLS_BYTES);
         const uint32_t out_s = sbase + (uint32_t)(SMEM_OUT + ew * OUT_PER_WARP);   // 1024-aligned
         // a drained TMEM region goes back to the CTA that issues the MMAs
         auto release_region = [&](uint32_t r) {
@@ -817,6 +1270,42 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
         };
         uint32_t job = 0;
         bool ok = true;
+        if constexpr (!GENERAL) {
+            FragTile ft;
+            ft.bar0 = bar0;
+            ft.abort_flag = abort_flag;
+            ft.tmem = lane_base;
+            ft.out_s = out_s;
+            ft.quad = quad;
+            ft.lane = lane;
+            ft.cgrp = cgrp;
+            ft.tile = 0;
+            // RUNS: a buffer per warp; else two per column half, in turn
+            ft.colc = reinterpret_cast<float4*>(smem + SMEM_COLS + (EPI == EPI_RUNS ? ew : 2 * cgrp) * COLS_BYTES);
+            auto place = [&](int u) {
+                ft.m0 = (int64_t)tile_m(u) * BM + quad * 32;
+                ft.nc0 = tile_n(u) * BN + cgrp * EPI_COLS;
+            };
+            if constexpr (EPI == EPI_RUNS) {
+                for (int u = first_u; u < n_units && ok; u += step_u) {
+                    place(u);
+                    ok = runs_tile<BNT, PAIR>(p, ft, job, release_region);
+                }
+            } else if (first_u < n_units) {
+                const ColPlan<EPI> cp(p);
+                ColLoad cl;
+                place(first_u);
+                cl.load(p, cp, ft, EPI_COLS);
+                cl.store<C>(cp, ft);
+                for (int u = first_u; u < n_units && ok; u += step_u, ++ft.tile) {
+                    place(u + step_u);               // (coordinates only)
+                    FragTile nxt = ft;
+                    if (u + step_u >= n_units) nxt.nc0 = -1;
+                    place(u);
+                    ok = frag_tile<EPI, ROWS, BNT, PAIR, OUT>(p, cp, ft, nxt, cl, job, release_region);
+                }
+            }
+        } else
         for (int u = first_u; u < n_units && ok; u += step_u) {
             const int64_t m0 = (int64_t)tile_m(u) * BM;
             const int nc0 = tile_n(u) * BN + cgrp * EPI_COLS;    // this warp's first column
@@ -839,14 +1328,6 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
             if (m < p.M) {
                 sa0 = p.s_a_per_row ? __ldg(p.s_a + m * 2) : __ldg(p.s_a);
                 sa1 = p.s_a_per_row ? __ldg(p.s_a + m * 2 + 1) : __ldg(p.s_a + 1);
-            }
-            if constexpr (GENERAL && BN == REGION) {
-                if (p.runs) {
-                    if (!runs_tile(p, sbase, bar0, abort_flag, lane_base, out_s, reinterpret_cast<float*>(colc), lane,
-                                   quad, m, m0, nc0, job))
-                        ok = false;
-                    continue;
-                }
             }
             // part: the exact accumulator of the first group (or the running
             // sum of the segments of the tile's only group)
@@ -895,10 +1376,10 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                 }
                 // the final job: finish the tile's outputs, 8 columns at a time
                 const float sc = p.g[g_last].acc_scale;
-                const bool dbg = GENERAL && p.acc_dbg != nullptr && m < p.M;
-                constexpr bool has_next = NEXT;
-                const bool y_tma = GENERAL ? p.y_tma != 0 : true;
-                const bool write_y = (GENERAL || NEXT) ? p.write_y != 0 : true;
+                const bool dbg = p.acc_dbg != nullptr && m < p.M;
+                constexpr bool has_next = EPI == EPI_GENERAL_NEXT;
+                const bool y_tma = p.y_tma != 0;
+                const bool write_y = p.write_y != 0;
                 // fp16 outputs go through the staging tile for the TMA store and
                 // for the next layer's quantizer
                 const bool staged_out = y_tma || has_next;
@@ -972,12 +1453,12 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
                         bulk_commit();
                     }
                 }
-                if constexpr (BN == REGION) {
-                    if (has_next && m < p.M) next_layer_codes(p, out_s, lane, m, nc0);
+                if constexpr (has_next) {
+                    if (m < p.M) next_layer_codes(p, out_s, lane, m, nc0);
                 }
             }
         }
-        if (((GENERAL || NEXT) ? p.y_tma && p.write_y : true) && lane == 0) bulk_wait0();   // stores complete before the CTA exits
+        if (OUT != OUT_BATCH && p.y_tma && p.write_y && lane == 0) bulk_wait0();   // stores complete before the CTA exits
     }
 
     tc_fence_before();
@@ -1028,6 +1509,83 @@ bool encode_rows(EncodeTiledFn enc, CUtensorMap* map, const uint8_t* base, int64
                CU_TENSOR_MAP_INTERLEAVE_NONE, KSTAGE == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B,
                CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// ---- kernel variants ---------------------------------------------------------
+
+struct Variant {
+    int epi;
+    bool rows;       // activation scales per row (LEAN, NEXT; the others take either)
+    bool f4;
+    int bn;
+    bool pair;
+    int out;
+    int smem;
+    void (*fn)(SParams);
+};
+
+template <int EPI, bool ROWS, int BNT, bool PAIR, int OUT>
+constexpr Variant make_variant() {
+    return Variant{EPI, ROWS, BNT == BN_F4, BNT, PAIR, OUT, Cfg<BNT, PAIR, OUT>::SMEM_ALLOC,
+                   staged_mma_kernel<EPI, ROWS, BNT, PAIR, OUT>};
+}
+
+const Variant kVariants[] = {
+    make_variant<EPI_LEAN, false, 256, true, OUT_BATCH>(),  make_variant<EPI_LEAN, true, 256, true, OUT_BATCH>(),
+    make_variant<EPI_LEAN, false, 256, false, OUT_BATCH>(), make_variant<EPI_LEAN, true, 256, false, OUT_BATCH>(),
+    make_variant<EPI_LEAN, false, 256, false, OUT_TMA>(),   make_variant<EPI_LEAN, true, 256, false, OUT_TMA>(),
+    make_variant<EPI_LEAN, false, 128, false, OUT_BATCH>(), make_variant<EPI_LEAN, true, 128, false, OUT_BATCH>(),
+    make_variant<EPI_LEAN, false, 64, false, OUT_BATCH>(),  make_variant<EPI_LEAN, true, 64, false, OUT_BATCH>(),
+    make_variant<EPI_LEAN, false, 240, true, OUT_BATCH>(),  make_variant<EPI_LEAN, true, 240, true, OUT_BATCH>(),
+    make_variant<EPI_LEAN, false, 240, false, OUT_BATCH>(), make_variant<EPI_LEAN, true, 240, false, OUT_BATCH>(),
+    make_variant<EPI_SEG, true, 256, true, OUT_BATCH>(),    make_variant<EPI_SEG, true, 256, false, OUT_BATCH>(),
+    make_variant<EPI_SEG, true, 128, false, OUT_BATCH>(),   make_variant<EPI_SEG, true, 240, true, OUT_BATCH>(),
+    make_variant<EPI_SEG, true, 240, false, OUT_BATCH>(),   make_variant<EPI_NEXT, false, 256, false, OUT_TMA>(),
+    make_variant<EPI_NEXT, true, 256, false, OUT_TMA>(),    make_variant<EPI_RUNS, true, 128, false, OUT_BATCH>(),
+    make_variant<EPI_RUNS, true, 64, false, OUT_BATCH>(),   make_variant<EPI_GENERAL, true, 256, false, OUT_GENERAL>(),
+    make_variant<EPI_GENERAL, true, 240, false, OUT_GENERAL>(),
+    make_variant<EPI_GENERAL_NEXT, true, 256, false, OUT_GENERAL>(),
+};
+constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
+
+// SM cycles of one tile: max(stages * stage + fixed, epilogue).  Fitted to timed calls
+// (one GB300, 1.93 GHz; M x K x N, variant: us): 8192 x 4096 x 4096 pair 109, 256 120,
+// 256 TMA 132, 128 156, 64 259; 16384 x 768 x 3072 pair 82, 256 73, 256 TMA 66, 128 79,
+// 64 117; 2048 x 4096 x 11008 pair 83, 256 92, 128 116; 512 x 4096 x 4096 pair 28, 256 26,
+// 128 23, 64 31; 300 x 4096 x 1024 pair 23, 256 21, 128 17, 64 16.  (An MMA takes about 110
+// cycles however narrow, so 64 columns pay only where 128 leave SMs idle.)
+struct TileCost {
+    double stage, fixed, epilogue;
+};
+TileCost tile_cost(const Variant& v) {
+    if (v.pair) return {560.0, 2500.0, 11500.0};
+    if (v.bn > 128) return v.out == OUT_TMA ? TileCost{700.0, 2300.0, 8800.0} : TileCost{640.0, 2500.0, 10200.0};
+    if (v.bn > 64) return {420.0, 1800.0, 5000.0};
+    return {400.0, 1200.0, 3500.0};
+}
+
+// The variant of an epilogue with the shortest modelled time, whole waves of
+// tiles; tma: outputs can leave by TMA stores.
+const Variant* pick_variant(int epi, bool rows, bool f4, bool tma, int64_t M, int64_t N, int stages) {
+    const Variant* best = nullptr;
+    double best_t = 0.0;
+    for (const Variant& v : kVariants) {
+        if (v.epi != epi || v.f4 != f4) continue;
+        if ((epi == EPI_LEAN || epi == EPI_NEXT) && v.rows != rows) continue;
+        if (epi == EPI_LEAN && v.out == OUT_TMA && !tma) continue;
+        const int64_t mt = (M + BM - 1) / BM, nt = (N + v.bn - 1) / v.bn;
+        const int64_t slots = v.pair ? num_sms() / 2 : num_sms();
+        const int64_t units = v.pair ? (mt + 1) / 2 * nt : mt * nt;
+        const int64_t waves = (units + slots - 1) / (slots > 0 ? slots : 1);
+        const TileCost c = tile_cost(v);
+        const double mma = stages * c.stage + c.fixed;
+        const double t = (double)waves * (mma > c.epilogue ? mma : c.epilogue);
+        if (best == nullptr || t < best_t) {
+            best = &v;
+            best_t = t;
+        }
+    }
+    return best;
 }
 
 int64_t align1k(int64_t x) { return (x + 1023) / 1024 * 1024; }
@@ -1117,7 +1675,6 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     // add more than 7 % of padded columns (N = 256 would take two tiles)
     const bool f4_ok = a.next == nullptr && (int64_t)((a.N + BN_F4 - 1) / BN_F4) * BN_F4 * 100 <= (int64_t)a.N * 107;
     if (!staged_plan(geo, &sp, f4_ok)) return cudaErrorNotSupported;
-    const int tile_n = sp.f4 ? BN_F4 : BN;
     const int64_t rows_a = a.M;
     if ((int64_t)scratch_bytes < staged_scratch_bytes(geo, rows_a, a.N) || scratch == nullptr ||
         (uintptr_t)scratch % 256 != 0)
@@ -1189,7 +1746,20 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     memset(&p, 0, sizeof(p));
     EncodeTiledFn enc = encode_fn();
     if (enc == nullptr) return cudaErrorNotSupported;
-    if (!encode_rows(enc, &p.tma_a, xa, sp.eb, rows_a, BM) || !encode_rows(enc, &p.tma_b, xw, sp.eb, a.N, tile_n))
+    // ---- epilogue, tile width and pairing ----
+    const bool runs = geo.sub_k > 0, wr_y = a.Y != nullptr, has_next = a.next != nullptr;
+    const bool general = !runs && (a.acc_dbg != nullptr || (!wr_y && !has_next) ||
+                                   (a.flags & SONIQ_FLAG_TEST_DROP_ARRIVE) != 0 || (has_next && sp.seg_group >= 0));
+    const int epi = runs ? EPI_RUNS
+                    : general ? (has_next ? EPI_GENERAL_NEXT : EPI_GENERAL)
+                    : has_next ? EPI_NEXT
+                    : sp.seg_group >= 0 ? EPI_SEG : EPI_LEAN;
+    const Variant* var = pick_variant(epi, a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0, a.M, a.N, (int)(sp.eb / KSTAGE));
+    if (var == nullptr) return cudaErrorNotSupported;
+    const int tile_n = var->bn;
+    const bool pair = var->pair;
+    if (!encode_rows(enc, &p.tma_a, xa, sp.eb, rows_a, BM) ||
+        !encode_rows(enc, &p.tma_b, xw, sp.eb, a.N, pair ? tile_n / 2 : tile_n))
         return cudaErrorInvalidValue;
     p.s_a = a.s_a;
     p.s_w = a.s_w;
@@ -1222,14 +1792,15 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     }
     // outputs through TMA stores when the row pitch allows a tensor map (N * 2 bytes a multiple of 16)
     p.y_tma = 0;
-    if (p.write_y && a.N % 8 == 0 && (uintptr_t)a.Y % 16 == 0) {
+    if (var->out != OUT_BATCH && p.write_y && a.N % 8 == 0 && (uintptr_t)a.Y % 16 == 0) {
         cuuint64_t dims[2] = {(cuuint64_t)a.N, (cuuint64_t)a.M};
         cuuint64_t strides[1] = {(cuuint64_t)a.N * 2};
-        // 64 x 32 boxes, 128-byte swizzled; 240-column tiles (120 columns per warp) use 8 x 32 boxes
-        cuuint32_t box[2] = {sp.f4 ? 8u : 64u, 32u};
+        // 64 x 32 boxes, 128-byte swizzled, where a warp's columns are whole boxes; else 8 x 32 boxes
+        const bool box8 = tile_n / (NUM_EPI_WARPS / 4) % 64 != 0;
+        cuuint32_t box[2] = {box8 ? 8u : 64u, 32u};
         cuuint32_t estr[2] = {1, 1};
         if (enc(&p.tma_y, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, a.Y, dims, strides, box, estr,
-                CU_TENSOR_MAP_INTERLEAVE_NONE, sp.f4 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, box8 ? CU_TENSOR_MAP_SWIZZLE_NONE : CU_TENSOR_MAP_SWIZZLE_128B,
                 CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
             return cudaErrorInvalidValue;
         p.y_tma = 1;
@@ -1252,37 +1823,14 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
         const double lw = ak == SONIQ_ACT_PM1 ? 1.0 : (double)(1 << (G.bits_w - 1));
         S.inv_levels = (float)(1.0 / (la * lw));
     }
-    // kernel instantiation: debug accumulators, outputs that cannot leave by
-    // TMA stores, or no outputs at all take the general epilogue
-    p.runs = geo.sub_k > 0 ? 1 : 0;
+    p.runs = runs ? 1 : 0;
     p.nb = geo.nb;
-    const bool general = a.acc_dbg != nullptr || p.runs || (p.write_y && !p.y_tma) ||
-                         (!p.write_y && !p.has_next) || p.drop_first;
-    // 2-SM pairs on 256 x 256 tiles: the lean epilogue on 256-column tiles, for
-    // rows of at least 3072 codes (launched as clusters of two; each CTA loads
-    // 128-row halves of the B tile).  A pair waits for the slower of its two
-    // epilogues before it reuses a TMEM region, so where the epilogue sets the
-    // pace (short K: the K = 768 MLP layer, 123 -> 138 us as pairs; the
-    // K = 2304 conv, even) and for the next-layer epilogue, whose drain is
-    // longer, one CTA takes one tile.
-    int64_t row_codes = 0;
-    for (int g = 0; g < 2; ++g) row_codes += geo.g[g].pw;
-    const bool pair = !general && !p.has_next && row_codes >= 3072;
     p.pair_tiles = ((p.m_tiles + 1) / 2) * p.n_tiles;
-    if (pair && !encode_rows(enc, &p.tma_b2, xw, sp.eb, a.N, tile_n / 2)) return cudaErrorInvalidValue;
-    void (*kern)(SParams) =
-        sp.f4 ? (general ? staged_mma_kernel<true, false, BN_F4, false>
-                 : pair  ? staged_mma_kernel<false, false, BN_F4, true>
-                         : staged_mma_kernel<false, false, BN_F4, false>)
-        : general ? (p.has_next ? staged_mma_kernel<true, true, BN, false> : staged_mma_kernel<true, false, BN, false>)
-                  : p.has_next ? staged_mma_kernel<false, true, BN, false>
-                  : pair       ? staged_mma_kernel<false, false, BN, true>
-                               : staged_mma_kernel<false, false, BN, false>;
-    static bool attr_done[64][8] = {};
-    static int max_pairs[64][2] = {};
+    static bool attr_done[64][kNumVariants] = {};
+    static int max_pairs[64][kNumVariants] = {};
     int dev = 0;
     cudaGetDevice(&dev);
-    const int kidx = sp.f4 ? (pair ? 7 : 4 + (general ? 1 : 0)) : pair ? 6 : (general ? 2 : 0) + (p.has_next ? 1 : 0);
+    const int kidx = (int)(var - kVariants);
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
@@ -1292,36 +1840,35 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[1].val.programmaticStreamSerializationAllowed = 1;
-    const int smem_alloc = pair ? pair_smem_alloc() : SMEM_ALLOC;
     cfg.blockDim = dim3(NUM_THREADS, 1, 1);
-    cfg.dynamicSmemBytes = smem_alloc;
+    cfg.dynamicSmemBytes = var->smem;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     if (!attr_done[dev][kidx]) {
-        if ((err = cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_alloc)) !=
+        if ((err = cudaFuncSetAttribute((const void*)var->fn, cudaFuncAttributeMaxDynamicSharedMemorySize, var->smem)) !=
             cudaSuccess)
             return err;
-        if ((err = prefer_max_shared((const void*)kern)) != cudaSuccess) return err;
+        if ((err = prefer_max_shared((const void*)var->fn)) != cudaSuccess) return err;
         if (pair) {
             // pairs that can be resident at once (one CTA per SM)
             cfg.gridDim = dim3(2 * (unsigned)num_sms() / 2, 1, 1);
             int n = 0;
-            if ((err = cudaOccupancyMaxActiveClusters(&n, (const void*)kern, &cfg)) != cudaSuccess) return err;
-            max_pairs[dev][sp.f4 ? 1 : 0] = n;
+            if ((err = cudaOccupancyMaxActiveClusters(&n, (const void*)var->fn, &cfg)) != cudaSuccess) return err;
+            max_pairs[dev][kidx] = n;
         }
         attr_done[dev][kidx] = true;
     }
     if (pair) {
-        int pairs = max_pairs[dev][sp.f4 ? 1 : 0];
+        int pairs = max_pairs[dev][kidx];
         if (pairs < 1) return cudaErrorNotSupported;
         if (pairs > p.pair_tiles) pairs = p.pair_tiles;
         cfg.gridDim = dim3(2 * (unsigned)pairs, 1, 1);
         cfg.numAttrs = 2;
-        if ((err = cudaLaunchKernelEx(&cfg, kern, p)) != cudaSuccess) return err;
+        if ((err = cudaLaunchKernelEx(&cfg, var->fn, p)) != cudaSuccess) return err;
     } else {
         const int grid = p.total_tiles < num_sms() ? p.total_tiles : num_sms();
-        if ((err = launch_pdl(kern, dim3((unsigned)grid), dim3(NUM_THREADS), (size_t)smem_alloc, st, p)) !=
+        if ((err = launch_pdl(var->fn, dim3((unsigned)grid), dim3(NUM_THREADS), (size_t)var->smem, st, p)) !=
             cudaSuccess)
             return err;
     }

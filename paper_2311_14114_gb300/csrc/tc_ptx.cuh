@@ -52,6 +52,16 @@ __device__ __forceinline__ void set_flag(uint32_t flag, int v) {
     asm volatile("st.volatile.shared.u32 [%0], %1;" ::"r"(flag), "r"(v) : "memory");
 }
 
+// True in one lane of the (fully active) warp.  The issuing warps run their
+// loops with every lane and put only the asynchronous instructions under this
+// predicate: their operands then stay in uniform registers, where a loop under
+// `lane == 0` moves each one there before every instruction.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t r;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+    return r != 0;
+}
+
 // Waits for phase `parity` of `bar` to complete.  Polls tightly and every 64
 // polls looks at the abort flag and the clock: gives up (false) when the CTA
 // is aborting, or after timeout_ns, in which case it records `err_bit` in the
@@ -74,6 +84,12 @@ __device__ __forceinline__ bool wait_bounded(uint32_t bar, uint32_t parity, uint
             }
         }
     }
+}
+
+// wait_bounded by a whole warp, with one result for all its lanes.
+__device__ __forceinline__ bool wait_bounded_warp(uint32_t bar, uint32_t parity, uint32_t abort_flag,
+                                                  long long timeout_ns, unsigned* err, unsigned err_bit) {
+    return __all_sync(0xffffffffu, wait_bounded(bar, parity, abort_flag, timeout_ns, err, err_bit)) != 0;
 }
 
 // 2-D tiled TMA load into shared memory, completing on `bar` (transaction bytes).
