@@ -184,7 +184,7 @@ struct ExpandParams {
     int32_t conv, H, W, P, Q, R, S, sh, sw, ph, pw;
     int32_t cpt[2];
     uint64_t cpt_magic[2];     // ceil(2^32 / cpt): tap = (kb * magic) >> 32, exact for kb < 2^32 / cpt
-    int32_t vec16[2];          // source blocks of the group can be read as 16-byte vectors
+    int32_t vec8[2];           // source blocks of the group can be read as 8-byte vectors
     // code encoding of each group: 0 unsigned, 1 n-bit two's complement (weights,
     // signed activations), 2 one-bit +-1 (bit 1 -> +1, bit 0 -> -1, positions
     // from count[g] on -> 0)
@@ -199,153 +199,479 @@ __device__ __forceinline__ uint32_t twos_to_e4m3(uint32_t x) {
     return (x & ~neg) | ((mag | 0x80808080u) & neg);
 }
 
-// This block's N packed words from src (16-byte loads when the group allows).
-template <int N>
-__device__ __forceinline__ void load_block_words(const uint8_t* src, bool vec16, uint32_t (&words)[N]) {
-    if constexpr (N % 4 == 0) {
-        if (vec16) {
-#pragma unroll
-            for (int i = 0; i < N; i += 4) {
-                const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + i / 4);
-                words[i] = v.x;
-                words[i + 1] = v.y;
-                words[i + 2] = v.z;
-                words[i + 3] = v.w;
+// The packed words that part `part` of PARTS equal parts of a block of N-bit
+// codes needs (8 / PARTS output words of code bytes): its words of the 4- and
+// 2-bit slices, the 1-bit slice's only word (N = 8: its own words).
+template <int N, int PARTS>
+struct PartWords {
+    static constexpr int TW = 8 / PARTS;              // output words (four codes each)
+    uint32_t w8[N == 8 ? TW : 1], w4[TW >= 2 ? TW / 2 : 1], w2[TW > 4 ? 2 : 1], w1;
+
+    // from the block at src: src.one(i) is its word i, src.two(i) words i and i + 1
+    // where vec8 (8-byte aligned)
+    template <typename Src>
+    __device__ __forceinline__ void load(const Src& src, int part, bool vec8) {
+        if constexpr (N == 8) {
+            pair_loads<TW>(src, part * TW, vec8, w8);
+        } else {
+            if constexpr ((N & 4) != 0) pair_loads<TW / 2>(src, part * (TW / 2), vec8, w4);
+            constexpr int at2 = N & 4;
+            if constexpr ((N & 2) != 0) {
+                if constexpr (PARTS == 1) pair_loads<2>(src, at2, false, w2);
+                else w2[0] = src.one(at2 + (PARTS == 2 ? part : part >> 1));
             }
-            return;
+            constexpr int at1 = (N & 4) + (N & 2);
+            if constexpr ((N & 1) != 0) w1 = src.one(at1);
         }
     }
+    __device__ __forceinline__ void zero() {
 #pragma unroll
-    for (int i = 0; i < N; ++i) words[i] = __ldg(reinterpret_cast<const uint32_t*>(src) + i);
+        for (int i = 0; i < (N == 8 ? TW : 1); ++i) w8[i] = 0u;
+#pragma unroll
+        for (int i = 0; i < (TW >= 2 ? TW / 2 : 1); ++i) w4[i] = 0u;
+#pragma unroll
+        for (int i = 0; i < (TW > 4 ? 2 : 1); ++i) w2[i] = 0u;
+        w1 = 0u;
+    }
+    // byte b of o[k]: the pattern of code 4 (TW part + k) + b
+    __device__ __forceinline__ void bytes(int part, uint32_t (&o)[TW]) const {
+#pragma unroll
+        for (int k = 0; k < TW; ++k) {
+            if constexpr (N == 8) {
+                o[k] = w8[k];
+            } else {
+                uint32_t v = 0u;
+                if constexpr ((N & 4) != 0) v |= (w4[k >> 1] >> (4 * (k & 1))) & 0x0F0F0F0Fu;
+                if constexpr ((N & 2) != 0) {
+                    const uint32_t w = PARTS == 1 ? w2[k >> 2] : (PARTS == 2 ? w2[0] : w2[0] >> (4 * (part & 1)));
+                    v |= ((w >> (2 * (k & 3))) & 0x03030303u) << (N & 4);
+                }
+                if constexpr ((N & 1) != 0)
+                    v |= (((PARTS == 1 ? w1 : w1 >> (TW * part)) >> k) & 0x01010101u) << ((N & 4) + (N & 2));
+                o[k] = v;
+            }
+        }
+    }
+
+private:
+    template <int C, typename Src, int D>
+    __device__ __forceinline__ static void pair_loads(const Src& src, int at, bool vec8, uint32_t (&w)[D]) {
+        if constexpr (C % 2 == 0 && C > 0) {
+            if (vec8) {
+#pragma unroll
+                for (int i = 0; i < C; i += 2) {
+                    const uint2 v = src.two(at + i);
+                    w[i] = v.x;
+                    w[i + 1] = v.y;
+                }
+                return;
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < C; ++i) w[i] = src.one(at + i);
+    }
+};
+
+struct GlobalWords {
+    const uint32_t* p;
+    __device__ __forceinline__ explicit GlobalWords(const uint8_t* src) : p(reinterpret_cast<const uint32_t*>(src)) {}
+    __device__ __forceinline__ uint32_t one(int i) const { return __ldg(p + i); }
+    __device__ __forceinline__ uint2 two(int i) const { return __ldg(reinterpret_cast<const uint2*>(p + i)); }
+};
+struct SharedWords {
+    uint32_t addr;
+    __device__ __forceinline__ uint32_t one(int i) const {
+        uint32_t v;
+        asm("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr + 4u * (uint32_t)i));
+        return v;
+    }
+    __device__ __forceinline__ uint2 two(int i) const {
+        uint2 v;
+        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr + 4u * (uint32_t)i));
+        return v;
+    }
+};
+
+// 16 bytes of operands from the words of part `part` of block kb (of group g).
+template <int N, int PARTS>
+__device__ __forceinline__ uint4 encode_piece(const ExpandParams& p, const PartWords<N, PARTS>& w, int g, int ck, int kb,
+                                              int part, __half2 bias, int32_t& csum) {
+    uint32_t o[PartWords<N, PARTS>::TW];
+    w.bytes(part, o);
+    if constexpr (PARTS == 1) {
+        // E2M1, two codes per byte (the first in the low nibble): a code c with
+        // |c| <= 4 is sign << 3 | |c|, the value c / 2
+        uint32_t y[8];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            uint32_t x = o[t];
+            if (ck == 1) {
+                // two's complement to sign << 3 | |c|: of one bit, 1 is -1; of two, 01 is 1, 11 -1, 10 -2
+                if constexpr (N == 1) x |= x << 3;
+                else x = ((x << 2) & 0x08080808u) | (x & ~(x << 1) & 0x02020202u) | (x & 0x01010101u);
+            }
+            y[t] = x | (x >> 4);                                        // bytes 0 and 2: two codes each
+        }
+        return make_uint4(__byte_perm(y[0], y[1], 0x6420u), __byte_perm(y[2], y[3], 0x6420u),
+                          __byte_perm(y[4], y[5], 0x6420u), __byte_perm(y[6], y[7], 0x6420u));
+    } else if constexpr (PARTS == 2) {
+        if (ck == 1) {
+#pragma unroll
+            for (int t = 0; t < 4; ++t) o[t] = twos_to_e4m3<N>(o[t]);
+        } else if (ck == 2) {
+            // one-bit +-1: bit 1 -> E4M3 +2^-9 (0x01), bit 0 -> -2^-9 (0x81); none past count
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int valid = p.count[g] - (kb * 32 + 16 * part + 4 * t);
+                const uint32_t keep = valid >= 4 ? 0xFFFFFFFFu : (valid <= 0 ? 0u : (1u << (8 * valid)) - 1u);
+                o[t] = (0x81818181u - (o[t] & 0x01010101u) * 0x80u) & keep;
+            }
+        }
+        return make_uint4(o[0], o[1], o[2], o[3]);
+    } else {
+        uint32_t h[4];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+            // signed codes: offset binary j + 2^(n-1); unsigned: the code u
+            const uint32_t x = ck == 1 ? (o[t] ^ (0x01010101u << (N - 1))) : o[t];
+            if (p.is_weight) csum += (int32_t)__dp4a(x, 0x01010101u, 0u);
+            uint32_t lo, hi;
+            bytes_to_magic_half2(x, lo, hi);
+            h[2 * t] = half2_sub(lo, bias);
+            h[2 * t + 1] = half2_sub(hi, bias);
+        }
+        return make_uint4(h[0], h[1], h[2], h[3]);
+    }
 }
 
-template <int N>
-__device__ __forceinline__ void expand_row(const ExpandParams& p, int64_t r, int g, int lane) {
-    const int kind = p.kind[g];
-    const bool vec16 = p.vec16[g] != 0;
-    const uint64_t magic = p.cpt_magic[g];
-    uint8_t* drow = p.dst + r * p.dst_row_bytes + p.dst_off[g];
-    int64_t img = 0;
-    int hp = 0, wq = 0;
-    if (p.conv) {
-        const int64_t pq = (int64_t)p.P * p.Q;
-        img = r / pq;
-        const int rem = (int)(r - img * pq);
-        const int pp = rem / p.Q, qq = rem - pp * p.Q;
-        hp = pp * p.sh - p.ph;
-        wq = qq * p.sw - p.pw;
-    }
-    const uint32_t flip = 0x01010101u << (N - 1);
+constexpr int kExpandRows = 4;      // rows a warp expands together
+
+// Rows r0 .. r0 + 3 (as far as they exist) of group g, by one warp; one
+// 16-byte piece of an expanded row per lane.
+//
+// Bound by L2 traffic (each packed byte read, each operand byte written once)
+// and by the latency of the loads.  A lane forms 16 output bytes (16 codes of
+// E4M3, 8 of fp16, 32 of E2M1) from the words that hold them, so every store
+// instruction writes 512 contiguous bytes; a whole block per lane wrote each
+// 32-byte sector in two instructions.  Four rows keep that many independent
+// loads in flight and share the index arithmetic.  Convolutions (64 x 56 x 56 x 64, 3 x 3,
+// 282 MB of operands: 192 us a call with one row per warp, 155 with four; 64 x 14 x 14 x 256
+// 29.7 and 29.2) and rows that expand_stream_kernel does not take.
+template <int N, int PARTS>
+__device__ __forceinline__ void expand_rows(const ExpandParams& p, int64_t r0, int g, int lane) {
+    using Words = PartWords<N, PARTS>;
+    constexpr int TW = Words::TW;
+    const bool vec8 = p.vec8[g] != 0;
     const int ck = p.code_kind[g];
+    const int nr = (int)(p.rows - r0 < kExpandRows ? p.rows - r0 : kExpandRows);
+    uint8_t* drow = p.dst + r0 * p.dst_row_bytes + p.dst_off[g];
+    const uint8_t* srow[kExpandRows];     // the row's group (conv: its image's)
+    int hp[kExpandRows], wq[kExpandRows];
+#pragma unroll
+    for (int i = 0; i < kExpandRows; ++i) {
+        const int64_t r = r0 + (i < nr ? i : 0);
+        hp[i] = wq[i] = 0;
+        if (!p.conv) {
+            srow[i] = p.src + r * p.src_row_bytes + p.src_off[g];
+        } else {
+            const uint32_t pq = (uint32_t)p.P * (uint32_t)p.Q, ru = (uint32_t)r;      // rows < 2^31
+            const uint32_t img = ru / pq, rem = ru - img * pq, pp = rem / (uint32_t)p.Q;
+            hp[i] = (int)pp * p.sh - p.ph;
+            wq[i] = (int)(rem - pp * (uint32_t)p.Q) * p.sw - p.pw;
+            srow[i] = p.src + (int64_t)img * p.H * p.W * p.src_row_bytes + p.src_off[g];
+        }
+    }
     const __half2 bias = __half2half2(__ushort_as_half(
         (unsigned short)(0x6400u + (ck == 1 ? (1u << (N - 1)) : (uint32_t)p.center[g]))));
-    int32_t csum = 0;
-    for (int kb = lane; kb < p.blk_dst[g]; kb += 32) {
-        const uint8_t* src = nullptr;
+    int32_t csum[kExpandRows];
+#pragma unroll
+    for (int i = 0; i < kExpandRows; ++i) csum[i] = 0;
+    const int pieces = p.blk_dst[g] * PARTS;
+    for (int c = lane; c < pieces; c += 32) {
+        const int kb = c / PARTS, part = c % PARTS;
+        Words w[kExpandRows];
         if (!p.conv) {
-            if (kb < p.blk_src[g]) src = p.src + r * p.src_row_bytes + p.src_off[g] + kb * 4 * N;
+            const bool in = kb < p.blk_src[g];
+#pragma unroll
+            for (int i = 0; i < kExpandRows; ++i) {
+                if (in) w[i].load(GlobalWords(srow[i] + kb * 4 * N), part, vec8);
+                else w[i].zero();
+            }
         } else {
-            const int tap = (int)(((uint64_t)kb * magic) >> 32);
+            const int tap = (int)(((uint64_t)kb * p.cpt_magic[g]) >> 32);
             const int cb = kb - tap * p.cpt[g];
-            if (tap < p.R * p.S) {
-                const int rr = tap / p.S, ss = tap - rr * p.S;
-                const int h = hp + rr, w = wq + ss;
-                if (h >= 0 && h < p.H && w >= 0 && w < p.W)
-                    src = p.src + ((img * p.H + h) * p.W + w) * p.src_row_bytes + p.src_off[g] + cb * 4 * N;
+            const int rr = tap / p.S, ss = tap - rr * p.S;
+            const bool in = tap < p.R * p.S;
+#pragma unroll
+            for (int i = 0; i < kExpandRows; ++i) {
+                const int h = hp[i] + rr, x = wq[i] + ss;
+                if (in && h >= 0 && h < p.H && x >= 0 && x < p.W)
+                    w[i].load(GlobalWords(srow[i] + ((int64_t)h * p.W + x) * p.src_row_bytes + cb * 4 * N), part,
+                              vec8);
+                else
+                    w[i].zero();
             }
         }
-        uint32_t words[N];
-        if (src != nullptr) {
-            load_block_words<N>(src, vec16, words);
-        } else {
 #pragma unroll
-            for (int i = 0; i < N; ++i) words[i] = 0u;
-        }
-        uint32_t o[8];
-        block_to_bytes<N>(words, o);
-        if (kind == 2) {
-            // E2M1, two codes per byte (the first in the low nibble): a code c with
-            // |c| <= 4 is sign << 3 | |c|, the value c / 2
-            uint32_t hw[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const uint32_t x = ck == 1 ? twos_to_e4m3<N>(o[t]) : o[t];   // sign in bit 7, magnitude below
-                const uint32_t nib = ((x >> 4) & 0x08080808u) | (x & 0x07070707u);
-                const uint32_t y = nib | (nib >> 4);                        // bytes 0 and 2: two codes each
-                hw[t >> 1] |= (__byte_perm(y, 0u, 0x0020u) & 0xFFFFu) << (16 * (t & 1));
-            }
-            *reinterpret_cast<uint4*>(drow + kb * 16) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        } else if (kind == 0) {
-            if (ck == 1) {
-#pragma unroll
-                for (int t = 0; t < 8; ++t) o[t] = twos_to_e4m3<N>(o[t]);
-            } else if (ck == 2) {
-                // one-bit +-1: bit 1 -> E4M3 +2^-9 (0x01), bit 0 -> -2^-9 (0x81); none past count
-#pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    const int valid = p.count[g] - (kb * 32 + 4 * t);
-                    const uint32_t keep = valid >= 4 ? 0xFFFFFFFFu : (valid <= 0 ? 0u : (1u << (8 * valid)) - 1u);
-                    o[t] = (0x81818181u - (o[t] & 0x01010101u) * 0x80u) & keep;
-                }
-            }
-            uint4* d = reinterpret_cast<uint4*>(drow + kb * 32);
-            d[0] = make_uint4(o[0], o[1], o[2], o[3]);
-            d[1] = make_uint4(o[4], o[5], o[6], o[7]);
-        } else {
-            uint32_t h[16];
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                // signed codes: offset binary j + 2^(n-1); unsigned: the code u
-                const uint32_t x = ck == 1 ? (o[t] ^ flip) : o[t];
-                if (p.is_weight) csum += (int32_t)__dp4a(x, 0x01010101u, 0u);
-                uint32_t lo, hi;
-                bytes_to_magic_half2(x, lo, hi);
-                h[2 * t] = half2_sub(lo, bias);
-                h[2 * t + 1] = half2_sub(hi, bias);
-            }
-            uint4* d = reinterpret_cast<uint4*>(drow + kb * 64);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) d[q] = make_uint4(h[4 * q], h[4 * q + 1], h[4 * q + 2], h[4 * q + 3]);
+        for (int i = 0; i < kExpandRows; ++i) {
+            const uint4 d = encode_piece<N, PARTS>(p, w[i], g, ck, kb, part, bias, csum[i]);
+            if (i < nr) *reinterpret_cast<uint4*>(drow + i * p.dst_row_bytes + (int64_t)c * 16) = d;
         }
     }
-    if (p.is_weight && kind == 1) {
+    if (PARTS == 4 && p.is_weight) {
         // sum of j over the row's group: the offset-binary sum minus 2^(n-1) per code
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) csum += __shfl_xor_sync(0xffffffffu, csum, o);
-        if (lane == 0) p.colsum[r * 2 + g] = csum - (1 << (N - 1)) * 32 * p.blk_dst[g];
+        for (int i = 0; i < kExpandRows; ++i) {
+            const int32_t s = __reduce_add_sync(0xffffffffu, csum[i]);
+            if (lane == 0 && i < nr) p.colsum[(r0 + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
+        }
     }
 }
 
-// Item `it` (row it / 2, group it % 2) of one operand.
+// Item `it` (rows 4 (it / 2) .. + 3, group it % 2) of one operand.
 __device__ __forceinline__ void expand_item(const ExpandParams& p, int64_t it, int lane) {
-    const int64_t r = it >> 1;
+    const int64_t r = (it >> 1) * kExpandRows;
     const int g = (int)(it & 1);
     if (p.blk_dst[g] == 0) return;
-    switch (p.bits[g]) {
-        case 1: expand_row<1>(p, r, g, lane); break;
-        case 2: expand_row<2>(p, r, g, lane); break;
-        case 3: expand_row<3>(p, r, g, lane); break;
-        case 4: expand_row<4>(p, r, g, lane); break;
-        case 5: expand_row<5>(p, r, g, lane); break;
-        case 6: expand_row<6>(p, r, g, lane); break;
-        case 7: expand_row<7>(p, r, g, lane); break;
-        default: expand_row<8>(p, r, g, lane); break;
+    if (p.kind[g] == 2) {
+        if (p.bits[g] == 1) expand_rows<1, 1>(p, r, g, lane);
+        else expand_rows<2, 1>(p, r, g, lane);
+    } else if (p.kind[g] == 0) {
+        switch (p.bits[g]) {
+            case 1: expand_rows<1, 2>(p, r, g, lane); break;
+            case 2: expand_rows<2, 2>(p, r, g, lane); break;
+            case 3: expand_rows<3, 2>(p, r, g, lane); break;
+            default: expand_rows<4, 2>(p, r, g, lane); break;
+        }
+    } else {
+        switch (p.bits[g]) {
+            case 1: expand_rows<1, 4>(p, r, g, lane); break;
+            case 2: expand_rows<2, 4>(p, r, g, lane); break;
+            case 3: expand_rows<3, 4>(p, r, g, lane); break;
+            case 4: expand_rows<4, 4>(p, r, g, lane); break;
+            case 5: expand_rows<5, 4>(p, r, g, lane); break;
+            case 6: expand_rows<6, 4>(p, r, g, lane); break;
+            case 7: expand_rows<7, 4>(p, r, g, lane); break;
+            default: expand_rows<8, 4>(p, r, g, lane); break;
+        }
     }
 }
 
-// Both operands in one launch: items 0 .. 2 rows_a - 1 are (row, group) of the
-// activations (pa), the rest of the weights (pw).
-__global__ void __launch_bounds__(256, 5) expand_kernel(const __grid_constant__ ExpandParams pa,
+// Both operands in one launch: items 0 .. items(pa) - 1 are (four rows, group)
+// of the activations, the rest of the weights (pw).
+__global__ void __launch_bounds__(256, 4) expand_kernel(const __grid_constant__ ExpandParams pa,
                                                      const __grid_constant__ ExpandParams pw) {
     tc::pdl_wait();   // launched with launch_pdl: the packed rows are written before this
     const int lane = threadIdx.x & 31;
     const int64_t warp_id = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    const int64_t items_a = pa.rows * 2;
-    for (int64_t item = warp_id; item < items_a + pw.rows * 2; item += nwarps) {
+    const int64_t items_a = (pa.rows + kExpandRows - 1) / kExpandRows * 2;
+    const int64_t items = items_a + (pw.rows + kExpandRows - 1) / kExpandRows * 2;
+    for (int64_t item = warp_id; item < items; item += nwarps) {
         if (item < items_a) expand_item(pa, item, lane);
         else expand_item(pw, item - items_a, lane);
     }
+}
+
+// The same for a linear layer, from packed rows staged in shared memory.
+//
+// With loads straight from global memory (expand_kernel) a warp waits for L2
+// once per 32 pieces, and the short kernel's straight-line code is fetched
+// cold: 20 us for the 8192 x 4096 x 4096 4/8-bit layer (94 MB moved), most stalls on
+// loads and on instruction fetch; streamed, 13 us.  Here a producer warp
+// streams tiles of eight packed rows (contiguous, so one bulk copy each)
+// through a ring; each consumer warp expands one row of a tile, two pieces per
+// step, with a short loop per group, and stores 512 contiguous bytes at a time.
+constexpr int kStreamWarps = 8;             // consumers: one row of a tile each
+constexpr int kStreamMaxStages = 6;
+constexpr size_t kStreamSmemPerSm = 216 * 1024;
+
+struct StreamParams {
+    ExpandParams op[2];       // activations, weights
+    unsigned* err;
+    int32_t stages, stage_bytes;
+    int32_t rpw;              // rows of a tile per warp
+};
+
+// One group of nr staged rows (row r's packed codes at src), by one warp.
+template <int N, int PARTS>
+__device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src, int64_t r, int nr, int g, int lane) {
+    const bool vec8 = p.vec8[g] != 0;
+    const int ck = p.code_kind[g];
+    const __half2 bias = __half2half2(__ushort_as_half(
+        (unsigned short)(0x6400u + (ck == 1 ? (1u << (N - 1)) : (uint32_t)p.center[g]))));
+    uint8_t* drow = p.dst + r * p.dst_row_bytes + p.dst_off[g];
+    const int pieces = p.blk_dst[g] * PARTS, have = p.blk_src[g] * PARTS;
+#pragma unroll 1
+    for (int i = 0; i < nr; ++i, src += (uint32_t)p.src_row_bytes, drow += p.dst_row_bytes) {
+        int32_t csum = 0;
+#pragma unroll 2
+        for (int c = lane; c < pieces; c += 32) {
+            const int kb = c / PARTS, part = c % PARTS;
+            PartWords<N, PARTS> w;
+            if (c < have) w.load(SharedWords{src + (uint32_t)(kb * 4 * N)}, part, vec8);
+            else w.zero();
+            reinterpret_cast<uint4*>(drow)[c] = encode_piece<N, PARTS>(p, w, g, ck, kb, part, bias, csum);
+        }
+        if (PARTS == 4 && p.is_weight) {
+            const int32_t s = __reduce_add_sync(0xffffffffu, csum);
+            if (lane == 0) p.colsum[(r + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
+        }
+    }
+}
+
+__global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kernel(const __grid_constant__ StreamParams sp) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ __align__(8) uint64_t full_bar[kStreamMaxStages], empty_bar[kStreamMaxStages];
+    __shared__ uint32_t abort_s, none_s;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t abort_flag = tc::smem_u32(&abort_s), base = tc::smem_u32(smem);
+    if (threadIdx.x == 0) {
+        for (int i = 0; i < sp.stages; ++i) {
+            tc::mbar_init(tc::smem_u32(&full_bar[i]), 1);
+            tc::mbar_init(tc::smem_u32(&empty_bar[i]), kStreamWarps);
+        }
+        tc::set_flag(abort_flag, 0);
+        none_s = 0u;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    tc::pdl_wait();      // launched with launch_pdl: the packed rows are written before this
+    // (no early trigger: GEMM CTAs that move in as this kernel's leave cost the MLP block 14 us)
+    const int tr = kStreamWarps * sp.rpw;                  // rows per tile
+    const int64_t tiles_a = (sp.op[0].rows + tr - 1) / tr;
+    const int64_t tiles = tiles_a + (sp.op[1].rows + tr - 1) / tr;
+    int b = 0;
+    uint32_t ph = 0u;
+    if (warp == kStreamWarps) {
+        // ---- producer ----
+        bool ok = true;
+        int64_t issued = 0;
+        for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, ++issued) {
+            if (issued >= sp.stages) {
+                ok = tc::wait_bounded_warp(tc::smem_u32(&empty_bar[b]), ph ^ 1u, abort_flag, kTimeoutNs, sp.err, kErrWait);
+                if (!ok) break;
+            }
+            const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
+            const int64_t r0 = (t < tiles_a ? t : t - tiles_a) * tr;
+            const int nr = (int)(p.rows - r0 < tr ? p.rows - r0 : tr);
+            const int bytes = nr * (int)p.src_row_bytes, body = bytes & ~15;
+            const uint8_t* src = p.src + r0 * p.src_row_bytes;      // 16-byte aligned: eight rows of 4-byte multiples
+            const uint32_t dst = base + (uint32_t)(b * sp.stage_bytes), bar = tc::smem_u32(&full_bar[b]);
+            if (lane == 0 && body > 0) {
+                asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(body)
+                             : "memory");
+                tc::bulk_load(dst, src, (uint32_t)body, bar);
+            }
+            // a last tile may end within 16 bytes
+            if (lane < (bytes - body) / 4)
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + body + 4 * lane),
+                             "r"(__ldg(reinterpret_cast<const uint32_t*>(src + body) + lane))
+                             : "memory");
+            __syncwarp();
+            if (lane == 0) tc::mbar_arrive(bar);
+            if (++b == sp.stages) {
+                b = 0;
+                ph ^= 1u;
+            }
+        }
+        // abandoned: the copies in flight land before the CTA exits
+        if (!ok && lane == 0)
+            for (int i = 0; i < sp.stages; ++i)
+                tc::wait_bounded(tc::smem_u32(&full_bar[i]), i < b ? ph : ph ^ 1u, tc::smem_u32(&none_s), kTimeoutNs,
+                                 sp.err, kErrWait);
+        return;
+    }
+    // ---- consumers ----
+    for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+        if (!tc::wait_bounded_warp(tc::smem_u32(&full_bar[b]), ph, abort_flag, kTimeoutNs, sp.err, kErrWait)) return;
+        const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
+        const int64_t r = (t < tiles_a ? t : t - tiles_a) * tr + warp * sp.rpw;
+        const int nr = p.rows - r < sp.rpw ? (int)(p.rows - r) : sp.rpw;
+        if (nr > 0) {
+            uint32_t row = base + (uint32_t)(b * sp.stage_bytes) + (uint32_t)(warp * sp.rpw * (int)p.src_row_bytes);
+            asm volatile("" : "+r"(row)::"memory");        // keeps the row's loads behind the wait
+#pragma unroll 1
+            for (int g = 0; g < 2; ++g) {
+                if (p.blk_dst[g] == 0) continue;
+                const uint32_t src = row + (uint32_t)p.src_off[g];
+                const int n = p.bits[g];
+                if (p.kind[g] == 2) {
+                    if (n == 1) stream_group<1, 1>(p, src, r, nr, g, lane);
+                    else stream_group<2, 1>(p, src, r, nr, g, lane);
+                } else if (p.kind[g] == 0) {
+                    switch (n) {
+                        case 1: stream_group<1, 2>(p, src, r, nr, g, lane); break;
+                        case 2: stream_group<2, 2>(p, src, r, nr, g, lane); break;
+                        case 3: stream_group<3, 2>(p, src, r, nr, g, lane); break;
+                        default: stream_group<4, 2>(p, src, r, nr, g, lane); break;
+                    }
+                } else {
+                    switch (n) {
+                        case 1: stream_group<1, 4>(p, src, r, nr, g, lane); break;
+                        case 2: stream_group<2, 4>(p, src, r, nr, g, lane); break;
+                        case 3: stream_group<3, 4>(p, src, r, nr, g, lane); break;
+                        case 4: stream_group<4, 4>(p, src, r, nr, g, lane); break;
+                        case 5: stream_group<5, 4>(p, src, r, nr, g, lane); break;
+                        case 6: stream_group<6, 4>(p, src, r, nr, g, lane); break;
+                        case 7: stream_group<7, 4>(p, src, r, nr, g, lane); break;
+                        default: stream_group<8, 4>(p, src, r, nr, g, lane); break;
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(tc::smem_u32(&empty_bar[b]));
+        if (++b == sp.stages) {
+            b = 0;
+            ph ^= 1u;
+        }
+    }
+}
+
+// expand_stream_kernel where its ring takes the rows; false where it does not
+// (convolutions gather their rows; packed rows off the 16-byte grid or too long).
+bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st, cudaError_t* err) {
+    if (a.conv || (uintptr_t)a.src % 16 != 0 || (uintptr_t)w.src % 16 != 0) return false;
+    const int64_t row = a.src_row_bytes > w.src_row_bytes ? a.src_row_bytes : w.src_row_bytes;
+    // four CTAs per SM, or two where four rings of two stages do not fit (rows over 3.4 KB;
+    // 8192 x 4096 x 4096 4/8 bits: two 101, three 99.7, four 99.4 us a call; 2/8 bits 81, 80, 79.6)
+    int per_sm = kStreamWarps * row * 2 + 256 <= (int64_t)kStreamSmemPerSm / 4 ? 4 : 2;
+    const int64_t smem_cta = (int64_t)kStreamSmemPerSm / per_sm;
+    // short rows: several per warp and stage (about 12 KB), as long as every CTA gets two tiles
+    // (16384 x 768 x 3072: 61 us a call, one row per warp 70)
+    const int64_t cap = (int64_t)num_sms() * per_sm, all = a.rows + w.rows;
+    int64_t rpw = 12 * 1024 / (kStreamWarps * row);
+    if (rpw > all / (2 * cap * kStreamWarps)) rpw = all / (2 * cap * kStreamWarps);
+    if (rpw > 4) rpw = 4;
+    if (rpw < 1) rpw = 1;
+    const int64_t tr = kStreamWarps * rpw;
+    const int64_t stage = (tr * row + 127) / 128 * 128;
+    const int64_t stages = smem_cta / stage;
+    if (stages < 2) return false;
+    StreamParams sp;
+    sp.op[0] = a;
+    sp.op[1] = w;
+    sp.err = device_error_word();
+    if (sp.err == nullptr) return false;
+    sp.stages = (int32_t)(stages < kStreamMaxStages ? stages : kStreamMaxStages);
+    sp.stage_bytes = (int32_t)stage;
+    sp.rpw = (int32_t)rpw;
+    const int64_t tiles = (a.rows + tr - 1) / tr + (w.rows + tr - 1) / tr;
+    static bool attr_done[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return false;
+    if (!attr_done[dev]) {
+        *err = cudaFuncSetAttribute(expand_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)kStreamSmemPerSm / 2);
+        if (*err == cudaSuccess) *err = prefer_max_shared((const void*)expand_stream_kernel);
+        if (*err != cudaSuccess) return true;
+        attr_done[dev] = true;
+    }
+    *err = launch_pdl(expand_stream_kernel, dim3((unsigned)(tiles < cap ? tiles : cap)), dim3((kStreamWarps + 1) * 32),
+                      (size_t)(sp.stages * sp.stage_bytes), st, sp);
+    return true;
 }
 
 // ---------------------------------------------------------------------------
@@ -1699,7 +2025,8 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
         e.center[g] = sp.g[g].center;
         e.cpt[g] = G.pa / 32 > 0 ? G.pa / 32 : 1;
         e.cpt_magic[g] = (((uint64_t)1 << 32) + (uint64_t)e.cpt[g] - 1) / (uint64_t)e.cpt[g];
-        e.vec16[g] = (G.a_off % 16 == 0 && geo.a_row_bytes % 16 == 0 && (uintptr_t)a.Ap % 16 == 0) ? 1 : 0;
+        // a block's parts start at multiples of 8 bytes where its words come in pairs (4-bit slices)
+        e.vec8[g] = (G.a_off % 8 == 0 && geo.a_row_bytes % 8 == 0 && (uintptr_t)a.Ap % 8 == 0 && G.bits_a % 2 == 0) ? 1 : 0;
         e.code_kind[g] = geo.act_kind[g];
         e.count[g] = G.count;
     }
@@ -1714,7 +2041,7 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     e.sh = a.sh; e.sw = a.sw; e.ph = a.ph; e.pw = a.pw;
     (void)taps;
     auto grid_for = [](int64_t items) {
-        int64_t ctas = (items + 7) / 8;                        // 8 warps per CTA, one (row, group) per warp
+        int64_t ctas = (items + 7) / 8;                        // 8 warps per CTA, one (four rows, group) per warp
         const int64_t cap = (int64_t)num_sms() * 16;
         return (int)(ctas < 1 ? 1 : (ctas > cap ? cap : ctas));
     };
@@ -1725,7 +2052,7 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
         w.src_off[g] = G.w_off;
         w.blk_src[g] = G.pw / 32;
         w.center[g] = 0;
-        w.vec16[g] = (G.w_off % 16 == 0 && geo.w_row_bytes % 16 == 0 && (uintptr_t)a.Wp % 16 == 0) ? 1 : 0;
+        w.vec8[g] = (G.w_off % 8 == 0 && geo.w_row_bytes % 8 == 0 && (uintptr_t)a.Wp % 8 == 0 && G.bits_w % 2 == 0) ? 1 : 0;
         w.code_kind[g] = geo.act_kind[g] == SONIQ_ACT_PM1 ? 2 : 1;
     }
     w.src = a.Wp;
@@ -1736,8 +2063,12 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     w.colsum = colsum;
     w.conv = 0;
     // activations and weights in one launch
-    cudaError_t err = launch_pdl(expand_kernel, dim3((unsigned)grid_for(rows_a * 2 + (int64_t)a.N * 2)), dim3(256), 0,
-                                 st, e, w);
+    cudaError_t err = cudaSuccess;
+    if (!launch_stream(e, w, st, &err))
+        err = launch_pdl(expand_kernel,
+                         dim3((unsigned)grid_for((rows_a + kExpandRows - 1) / kExpandRows * 2 +
+                                                 ((int64_t)a.N + kExpandRows - 1) / kExpandRows * 2)),
+                         dim3(256), 0, st, e, w);
     note_launch();
     if (err != cudaSuccess) return err;
 
