@@ -8,6 +8,27 @@
 
 namespace soniq {
 
+// ---- packed fp32 pairs -------------------------------------------------------
+// Two fp32 operations per instruction (each element rounded as its scalar
+// counterpart).  Products and sums are spelled as fused multiply-adds with
+// -0 and 1, which nothing can fuse further.
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    float2 d;
+    asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
+        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return fma2(a, b, make_float2(-0.0f, -0.0f)); }
+__device__ __forceinline__ float2 add2(float2 a, float b) { return fma2(a, make_float2(1.0f, 1.0f), make_float2(b, b)); }
+// a * b + c clamped to [0, 1]; NaN gives 0.
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {
+    float d;
+    asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(d) : "f"(a), "f"(b), "f"(c));
+    return d;
+}
+
 // ---- quantizers ------------------------------------------------------------
 // Both decide the integer code in fp32 with the operation order of the
 // paper's formulas: divide by the group scale (IEEE, round to nearest), then

@@ -108,6 +108,13 @@ cudaError_t launch_quantize_rows(const LayoutGeom& geo, const int32_t* perm, con
 bool quantize_gather_supported(const LayoutGeom& geo, int32_t scale_mode, const void* A);
 cudaError_t launch_quantize_gather(const LayoutGeom& geo, const int32_t* perm, const uint16_t* A, int64_t M,
                                    int32_t scale_mode, bool demote, float* s_a, uint8_t* Ap, cudaStream_t st);
+// Per-tensor scale, codes and packing in one cooperative launch of the same
+// kernel (rows streamed twice, the last ones kept on chip in between); `bar`,
+// `part` and `err_bit` as for launch_quantize_fused.  cudaErrorNotSupported
+// where launch_quantize_gather does not take the layout.
+cudaError_t launch_quantize_stream(const LayoutGeom& geo, const int32_t* perm, const uint16_t* A, int64_t M, float* s_a,
+                                   uint8_t* Ap, cudaStream_t st, unsigned* bar, float* part, int max_ctas,
+                                   unsigned err_bit);
 cudaError_t launch_weight_absmax(const LayoutGeom& geo, const int32_t* perm, const float* W,
                                  int32_t N, float* s_out, cudaStream_t st);
 cudaError_t launch_pack_weights(const LayoutGeom& geo, const int32_t* perm, const float* W,

@@ -871,19 +871,6 @@ __device__ __forceinline__ void frag_blocks(uint32_t taddr, F&& f) {
     frag_step<0, NCH>(taddr, first, f);
 }
 
-// Two fp32 operations per instruction (each element rounded as its scalar
-// counterpart).  Products and sums are spelled as fused multiply-adds with
-// -0 and 1, which nothing can fuse further.
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-    float2 d;
-    asm("{\n\t.reg .b64 x, y, z, w;\n\tmov.b64 x, {%2, %3};\n\tmov.b64 y, {%4, %5};\n\tmov.b64 z, {%6, %7};\n\t"
-        "fma.rn.f32x2 w, x, y, z;\n\tmov.b64 {%0, %1}, w;\n\t}"
-        : "=f"(d.x), "=f"(d.y)
-        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return fma2(a, b, make_float2(-0.0f, -0.0f)); }
-
 // Four 8 x 8 blocks of 16-bit values (rows 0..31 of the warp); lane l gives the address of row l.
 __device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&w)[4]) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]),
