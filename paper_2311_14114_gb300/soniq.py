@@ -116,13 +116,23 @@ def _check(status: int, where: str):
         raise SoniqError(status, where)
 
 
-def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
+    return None if t is None else t.data_ptr()
 
 
-def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+# The current stream's handle without building a torch.cuda.Stream, which takes
+# 2.8 us; a small layer makes two library calls of 3 to 4 us each.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _current(device_index: int) -> int:
+    if _raw_stream is None:
+        return torch.cuda.current_stream(device_index).cuda_stream
+    return _raw_stream(device_index)
+
+
+def _stream(stream=None) -> int:
+    return _current(torch.cuda.current_device()) if stream is None else stream.cuda_stream
 
 
 def _need(t: torch.Tensor, dtype, name: str):
@@ -143,11 +153,11 @@ _scratch = {}
 def _get_scratch(nbytes: int, device, stream, use: str) -> Optional[torch.Tensor]:
     if nbytes <= 0:
         return None
-    s = torch.cuda.current_stream(device) if stream is None else stream
-    key = (use, torch.device(device).index, s.cuda_stream)
+    index = device.index
+    key = (use, index, _current(index) if stream is None else stream.cuda_stream)
     buf = _scratch.get(key)
     if buf is None or buf.numel() < nbytes:
-        with torch.cuda.stream(s):
+        with torch.cuda.stream(torch.cuda.current_stream(device) if stream is None else stream):
             buf = torch.zeros(((nbytes + 255) // 256) * 256, dtype=torch.uint8, device=device)
         _scratch[key] = buf
     return buf
@@ -193,19 +203,20 @@ class Layout:
         self.perm = perm_t.to(device if device is not None else "cuda")
         host.perm = ctypes.c_void_p(self.perm.data_ptr())
         self.c = host
+        self.ref = ctypes.byref(host)
 
     def row_bytes(self, is_weight: bool = False, taps: int = 1) -> int:
-        v = lib().soniq_packed_row_bytes(ctypes.byref(self.c), int(is_weight), int(taps))
+        v = lib().soniq_packed_row_bytes(self.ref, int(is_weight), int(taps))
         if v < 0:
             raise SoniqError(1, "soniq_packed_row_bytes")
         return int(v)
 
     def group_codes(self, g: int, is_weight: bool = False, taps: int = 1) -> int:
-        return int(lib().soniq_group_codes(ctypes.byref(self.c), int(g), int(is_weight), int(taps)))
+        return int(lib().soniq_group_codes(self.ref, int(g), int(is_weight), int(taps)))
 
     def scale_runs(self) -> int:
         """Scale entries per (row, group): soniq_scale_runs."""
-        return int(lib().soniq_scale_runs(ctypes.byref(self.c)))
+        return int(lib().soniq_scale_runs(self.ref))
 
     def scale_shape(self, rows: Optional[int]) -> tuple:
         """Shape of a scale array: [rows][2] or [2], with a run axis when sub_k > 0."""
@@ -253,7 +264,7 @@ def pack_weights(layout: Layout, W: torch.Tensor, scale_mode: str = "row",
     if s_w is None:
         s_w = torch.empty(layout.scale_shape(N), dtype=torch.float32, device=W.device)
     mode = {"row": SCALE_PER_ROW, "tensor": SCALE_PER_TENSOR}[scale_mode]
-    _check(lib().soniq_pack_weights(ctypes.byref(layout.c), _ptr(W), N, taps, mode, _ptr(Wp),
+    _check(lib().soniq_pack_weights(layout.ref, _ptr(W), N, taps, mode, _ptr(Wp),
                                     _ptr(s_w), _stream(stream)), "soniq_pack_weights")
     return Wp, s_w
 
@@ -276,10 +287,10 @@ def quantize_act(layout: Layout, A: torch.Tensor, scale_mode: str = "tensor",
     if Ap is None:
         Ap = torch.empty((M, layout.row_bytes(False)), dtype=torch.uint8, device=A.device)
     if scratch is False:
-        need = int(lib().soniq_quantize_act_scratch_bytes(ctypes.byref(layout.c), M, mode))
+        need = int(lib().soniq_quantize_act_scratch_bytes(layout.ref, M, mode))
         scratch = _get_scratch(need, A.device, stream, "quantize")
     nbytes = 0 if scratch is None else scratch.numel() * scratch.element_size()
-    _check(lib().soniq_quantize_act(ctypes.byref(layout.c), _ptr(A), M, mode, _ptr(s_a), _ptr(Ap),
+    _check(lib().soniq_quantize_act(layout.ref, _ptr(A), M, mode, _ptr(s_a), _ptr(Ap),
                                     _ptr(scratch), nbytes, _stream(stream)), "soniq_quantize_act")
     return Ap, s_a
 
@@ -294,7 +305,7 @@ def quantize_act_oneshot(layout: Layout, A: torch.Tensor, s_a: Optional[torch.Te
         s_a = torch.empty((2,), dtype=torch.float32, device=A.device)
     if Ap is None:
         Ap = torch.empty((M, layout.row_bytes(False)), dtype=torch.uint8, device=A.device)
-    _check(lib().soniq_quantize_act_oneshot(ctypes.byref(layout.c), _ptr(A), M, _ptr(s_a), _ptr(Ap),
+    _check(lib().soniq_quantize_act_oneshot(layout.ref, _ptr(A), M, _ptr(s_a), _ptr(Ap),
                                             _stream(stream)), "soniq_quantize_act_oneshot")
     return Ap, s_a
 
@@ -312,9 +323,9 @@ def mp_gemm(layout: Layout, Ap: torch.Tensor, s_a: torch.Tensor, Wp: torch.Tenso
     od = OUT_BF16 if (Y is not None and Y.dtype == torch.bfloat16) or (Y is None and out_dtype == torch.bfloat16) \
         else OUT_F16
     qflags = int(flags) | (FLAG_FORCE_STAGED if next is not None else 0)
-    need = int(lib().soniq_mp_gemm_scratch_bytes(ctypes.byref(layout.c), M, N, qflags))
+    need = int(lib().soniq_mp_gemm_scratch_bytes(layout.ref, M, N, qflags))
     scratch = _get_scratch(need, Ap.device, stream, "gemm")
-    _check(lib().soniq_mp_gemm(ctypes.byref(layout.c), _ptr(Ap), _ptr(s_a), _SCALE[scale_mode], M,
+    _check(lib().soniq_mp_gemm(layout.ref, _ptr(Ap), _ptr(s_a), _SCALE[scale_mode], M,
                                _ptr(Wp), _ptr(s_w), N, _ptr(Y), od, _ptr(acc_dbg), int(flags),
                                _ptr(scratch), max(need, 0),
                                ctypes.byref(next.c) if next is not None else None, _stream(stream)),
@@ -324,8 +335,8 @@ def mp_gemm(layout: Layout, Ap: torch.Tensor, s_a: torch.Tensor, Wp: torch.Tenso
 
 def gemm_path(layout: Layout, M: int, N: int, flags: int = 0) -> str:
     """soniq_mp_gemm_path: the kernel soniq_mp_gemm runs for these arguments."""
-    need = max(int(lib().soniq_mp_gemm_scratch_bytes(ctypes.byref(layout.c), M, N, int(flags))), 0)
-    p = int(lib().soniq_mp_gemm_path(ctypes.byref(layout.c), M, N, int(flags), need))
+    need = max(int(lib().soniq_mp_gemm_scratch_bytes(layout.ref, M, N, int(flags))), 0)
+    p = int(lib().soniq_mp_gemm_path(layout.ref, M, N, int(flags), need))
     if p < 0:
         raise SoniqError(SONIQ_ERR_INVALID_ARG, "soniq_mp_gemm_path")
     return PATH_NAMES.get(p, str(p))
@@ -354,9 +365,9 @@ def mp_conv2d(layout: Layout, cd: CConvDesc, Xp: torch.Tensor, s_a: torch.Tensor
     od = OUT_BF16 if (Y is not None and Y.dtype == torch.bfloat16) or (Y is None and out_dtype == torch.bfloat16) \
         else OUT_F16
     qflags = int(flags) | (FLAG_FORCE_STAGED if next is not None else 0)
-    need = int(lib().soniq_mp_conv2d_scratch_bytes(ctypes.byref(layout.c), ctypes.byref(cd), qflags))
+    need = int(lib().soniq_mp_conv2d_scratch_bytes(layout.ref, ctypes.byref(cd), qflags))
     scratch = _get_scratch(need, Xp.device, stream, "gemm")
-    _check(lib().soniq_mp_conv2d(ctypes.byref(layout.c), ctypes.byref(cd), _ptr(Xp), _ptr(s_a),
+    _check(lib().soniq_mp_conv2d(layout.ref, ctypes.byref(cd), _ptr(Xp), _ptr(s_a),
                                  _SCALE[scale_mode], _ptr(Wp), _ptr(s_w), _ptr(Y), od,
                                  _ptr(acc_dbg), int(flags), _ptr(scratch), max(need, 0),
                                  ctypes.byref(next.c) if next is not None else None,
