@@ -128,7 +128,7 @@ enum {
 enum { SONIQ_OUT_F16 = 0, SONIQ_OUT_BF16 = 1 };
 
 enum {
-    SONIQ_FLAG_FORCE_GEMV = 1u,          /* soniq_mp_gemm: use the CUDA-core GEMV for any M <= 16 */
+    SONIQ_FLAG_FORCE_GEMV = 1u,          /* soniq_mp_gemm: use the GEMV for any M <= 16 */
     SONIQ_FLAG_FORCE_MMA = 2u,           /* soniq_mp_gemm: use a tensor-core kernel for any M */
     SONIQ_FLAG_FORCE_FUSED = 4u,         /* tensor-core work takes the fused kernel even when
                                             scratch for the staged path is given */
@@ -146,11 +146,13 @@ enum {
 
 /* Kernels behind soniq_mp_gemm (see soniq_mp_gemm_path). */
 enum {
-    SONIQ_PATH_GEMV = 0,           /* CUDA-core GEMV streaming the packed weights (small M) */
+    SONIQ_PATH_GEMV = 0,           /* GEMV streaming the packed weights (small M): dot products on CUDA
+                                      cores, or warp-level tensor instructions for M >= 3 */
     SONIQ_PATH_TENSOR = 1,         /* tcgen05 kernel expanding packed tiles on chip (no scratch) */
     SONIQ_PATH_TENSOR_STAGED = 2,  /* codes expanded once into scratch, then a tcgen05 GEMM */
-    SONIQ_PATH_TENSOR_SKINNY = 3   /* swap-AB tcgen05 kernel for few rows: packed weight rows
-                                      are the MMA's M = 128 side, converted on chip */
+    SONIQ_PATH_TENSOR_SKINNY = 3   /* few rows, packed weight rows converted on chip: warp-level
+                                      tensor instructions where the activation rows fit in shared
+                                      memory, else a swap-AB tcgen05 kernel */
 };
 /* Without flags, soniq_mp_gemm runs the GEMV for M <= SONIQ_GEMV_MAX_M and the
  * skinny tensor-core kernel for M <= SONIQ_SKINNY_MAX_M. */
@@ -329,8 +331,8 @@ SONIQ_API soniq_status soniq_quantize_act_oneshot(const soniq_layout *layout, co
  *   Acc_g[m][n] = sum over k in group g of u[m][k] * j[n][k]   (exact int32)
  *   Y[m][n]     = sum_g s_a(m,g) * s_w[n][g] / ((2^na_g - 1) * 2^(nw_g - 1)) * Acc_g[m][n]
  * computed in fp32 and rounded to nearest fp16 (or bf16).  M <= SONIQ_GEMV_MAX_M
- * runs a bandwidth-bound CUDA-core GEMV, M <= SONIQ_SKINNY_MAX_M the skinny
- * swap-AB tensor-core kernel, larger M the tcgen05 GEMM (flags can force a
+ * runs a GEMV over the packed weights, M <= SONIQ_SKINNY_MAX_M a skinny
+ * tensor-core kernel, larger M the tcgen05 GEMM (flags can force a
  * kernel; the GEMV takes M <= 16, the skinny kernel M <= 32);
  * soniq_mp_gemm_path tells which.
  *

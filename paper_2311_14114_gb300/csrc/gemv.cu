@@ -18,6 +18,7 @@
 
 #include "soniq_device.cuh"
 #include "soniq_internal.h"
+#include "tc_ptx.cuh"
 
 namespace soniq {
 namespace {
@@ -252,6 +253,7 @@ __global__ void __launch_bounds__(bulk_threads<MT>(), 1) gemv_bulk_kernel(const 
     }
     if (threadIdx.x < 32) rowsum[threadIdx.x] = 0;
     __syncthreads();
+    tc::pdl_wait();      // launched with launch_pdl: every global access comes after this
 
     bool ok = true;
     int round = 0;
@@ -424,9 +426,9 @@ cudaError_t run_bulk(const GemvParams& p, size_t smem, cudaStream_t st) {
     e = prefer_max_shared((const void*)gemv_bulk_kernel<MT>);
     if (e != cudaSuccess) return e;
     const int64_t grid = (p.N + p.rows_cta - 1) / p.rows_cta;
-    gemv_bulk_kernel<MT><<<(unsigned)grid, bulk_threads<MT>(), smem, st>>>(p);
-    note_launch();
-    return cudaGetLastError();
+    e = launch_pdl(gemv_bulk_kernel<MT>, dim3((unsigned)grid), dim3(bulk_threads<MT>()), smem, st, p);
+    if (e == cudaSuccess) note_launch();
+    return e;
 }
 
 }  // namespace

@@ -293,6 +293,7 @@ __global__ void __launch_bounds__(1024) quantize_fused_kernel(const FusedParams 
     __shared__ int abort_s;
     const int RH = p.row_halves;
     const int c0 = p.g[0].count, pa0 = p.g[0].pa;
+    tc::pdl_trigger();   // one wave of CTAs: the kernel that follows may be scheduled at once
     build_positions(pos_s, p.perm, p.K, c0, pa0);
     if (threadIdx.x == 0) abort_s = 0;
     __syncthreads();
@@ -609,6 +610,10 @@ __global__ void __launch_bounds__(kTileThreads, 1) quantize_tiles_kernel(const T
     const int c0 = p.g[0].count, pa0 = p.g[0].pa;
     const int KV = p.K >> 3;
     const int64_t tstep = (int64_t)gridDim.x * TR;
+    // launched with launch_pdl: every global access comes after this wait; one wave of CTAs,
+    // so the kernel that follows may be scheduled at once
+    tc::pdl_wait();
+    tc::pdl_trigger();
     // staging map: vector v of a tile is row v / KV, column v % KV; this thread
     // takes v = tid + u * blockDim for u < kTilePrefetch
     const int tile_vecs = TR * KV;
@@ -819,9 +824,9 @@ cudaError_t launch_quantize_rows(const LayoutGeom& geo, const int32_t* perm, con
     int64_t ctas = tensor_in_cta ? 1 : (M + tr - 1) / tr;
     const int64_t cap = (int64_t)num_sms();
     if (ctas > cap) ctas = cap;
-    quantize_tiles_kernel<<<(int)ctas, kTileThreads, smem, st>>>(p);
-    note_launch();
-    return cudaGetLastError();
+    const cudaError_t e = launch_pdl(quantize_tiles_kernel, dim3((unsigned)ctas), dim3(kTileThreads), smem, st, p);
+    if (e == cudaSuccess) note_launch();
+    return e;
 }
 
 // The one-pass per-tensor path, when every CTA's rows fit in shared memory

@@ -453,9 +453,16 @@ soniq_status soniq_mp_gemm(const soniq_layout* L, const uint8_t* Ap, const float
     const int path = gemm_path(geo, M, N, flags, scratch != nullptr ? scratch_bytes : 0);
     if (next != nullptr && path != SONIQ_PATH_TENSOR_STAGED) return SONIQ_ERR_UNSUPPORTED;
     if (path < 0) return path == -2 ? SONIQ_ERR_UNSUPPORTED : mma_check(geo);
-    if (path == SONIQ_PATH_GEMV) {
+    if (path == SONIQ_PATH_GEMV || path == SONIQ_PATH_TENSOR_SKINNY) {
         GemvArgs a{Ap, Wp, s_a, s_w, Y, acc_dbg, (int32_t)M, N, per_row, out_dtype == SONIQ_OUT_BF16};
-        return cuda_status(launch_gemv(geo, a, s));
+        // from three rows on, and where the rows fit on chip, warp-level tensor instructions
+        // (11008 x 4096 at 3/6 bits, us: M = 1 dot products 10.6 and 14.4; 2: 13.3, 14.7; 4: 16.4, 14.7;
+        // 12: 37, 16; 16 swap-AB tcgen05 kernel 33.5, 16.7; 32: 37, 23; 4096 x 4096 4/8 bits: M = 1 6.5, 7.5;
+        // 4: 8.2, 7.5; 16: 37, 8.9)
+        if (M >= 3 && rows_mma_supported(geo, M, N))
+            return cuda_status(launch_rows_mma(
+                geo, a, (flags & SONIQ_FLAG_TEST_DROP_ARRIVE) != 0 && path == SONIQ_PATH_TENSOR_SKINNY, s));
+        if (path == SONIQ_PATH_GEMV) return cuda_status(launch_gemv(geo, a, s));
     }
     if (path == SONIQ_PATH_TENSOR_STAGED && !aligned(scratch, 256)) return SONIQ_ERR_ALIGNMENT;
     MmaArgs a{};

@@ -149,6 +149,11 @@ struct GemvArgs {
 cudaError_t launch_gemv(const LayoutGeom& geo, const GemvArgs& a, cudaStream_t st);
 bool gemv_supported(const LayoutGeom& geo, int64_t M, int64_t N);
 
+// The same for M <= 32 rows on warp-level tensor instructions (rows_mma.cu); the
+// activation rows must fit in shared memory.  drop_first: the test hook.
+bool rows_mma_supported(const LayoutGeom& geo, int64_t M, int64_t N);
+cudaError_t launch_rows_mma(const LayoutGeom& geo, const GemvArgs& a, bool drop_first, cudaStream_t st);
+
 struct MmaArgs {
     const uint8_t* Ap;
     const uint8_t* Wp;
