@@ -1147,9 +1147,10 @@ __device__ __forceinline__ bool frag_tile(const SParams& p, const ColPlan<EPI>& 
 // Scale runs along K, one tile of an epilogue warp: every job is one run b of
 // one group g, whose exact integer sum is added in fp32 with its own scale,
 // y += (s_a(g, b) s_w(n, g, b) / (La Lw)) * Acc(g, b).  A job's scales are
-// loaded while the previous job is drained.  With debug accumulators, acc_dbg
-// receives [2][nb][M][N].  False after a wait ran out.
-template <int BNT, bool PAIR, typename Release>
+// loaded while the previous job is drained.  DBG: acc_dbg receives [2][nb][M][N]
+// (a run-time test per element, not taken, made a job's drain 2000 cycles instead
+// of 320).  False after a wait ran out.
+template <bool DBG, int BNT, bool PAIR, typename Release>
 __device__ __forceinline__ bool runs_tile(const SParams& p, const FragTile& t, uint32_t& job, Release&& release) {
     using C = Cfg<BNT, PAIR, OUT_BATCH>;
     constexpr int EPI_COLS = C::EPI_COLS, NCH = EPI_COLS / 8, NK = EPI_COLS / 32;
@@ -1198,7 +1199,7 @@ __device__ __forceinline__ bool runs_tile(const SParams& p, const FragTile& t, u
             for (int e = 0; e < 8; ++e) {
                 const float x = __fmul_rn(__uint_as_float(v[e]), sc);       // the exact integer sum
                 y[8 * c + e] = __fmaf_rn(__fmul_rn(s[e >> 1], k[e & 1]), x, y[8 * c + e]);
-                if (p.acc_dbg != nullptr) {
+                if constexpr (DBG) {
                     const int64_t m = t.m0 + 8 * (e >> 1) + (lane >> 2);
                     const int n = t.nc0 + 8 * c + 2 * (lane & 3) + (e & 1);
                     if (m < p.M && n < p.N) p.acc_dbg[(((int64_t)g * p.nb + b) * p.M + m) * p.N + n] = __float2int_rn(x);
@@ -1510,7 +1511,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
             if constexpr (EPI == EPI_RUNS) {
                 for (int u = first_u; u < n_units && ok; u += step_u) {
                     place(u);
-                    ok = runs_tile<BNT, PAIR>(p, ft, job, release_region);
+                    ok = runs_tile<ROWS, BNT, PAIR>(p, ft, job, release_region);
                 }
             } else if (first_u < n_units) {
                 const ColPlan<EPI> cp(p);
@@ -1736,7 +1737,7 @@ bool encode_rows(EncodeTiledFn enc, CUtensorMap* map, const uint8_t* base, int64
 
 struct Variant {
     int epi;
-    bool rows;       // activation scales per row (LEAN, NEXT; the others take either)
+    bool rows;       // activation scales per row (LEAN, NEXT); debug accumulators (RUNS)
     bool f4;
     int bn;
     bool pair;
@@ -1762,8 +1763,8 @@ const Variant kVariants[] = {
     make_variant<EPI_SEG, true, 256, true, OUT_BATCH>(),    make_variant<EPI_SEG, true, 256, false, OUT_BATCH>(),
     make_variant<EPI_SEG, true, 128, false, OUT_BATCH>(),   make_variant<EPI_SEG, true, 240, true, OUT_BATCH>(),
     make_variant<EPI_SEG, true, 240, false, OUT_BATCH>(),   make_variant<EPI_NEXT, false, 256, false, OUT_TMA>(),
-    make_variant<EPI_NEXT, true, 256, false, OUT_TMA>(),    make_variant<EPI_RUNS, true, 128, false, OUT_BATCH>(),
-    make_variant<EPI_RUNS, true, 64, false, OUT_BATCH>(),   make_variant<EPI_GENERAL, true, 256, false, OUT_GENERAL>(),
+    make_variant<EPI_NEXT, true, 256, false, OUT_TMA>(),    make_variant<EPI_RUNS, false, 128, false, OUT_BATCH>(),
+    make_variant<EPI_RUNS, false, 64, false, OUT_BATCH>(),  make_variant<EPI_RUNS, true, 64, false, OUT_BATCH>(),   make_variant<EPI_GENERAL, true, 256, false, OUT_GENERAL>(),
     make_variant<EPI_GENERAL, true, 240, false, OUT_GENERAL>(),
     make_variant<EPI_GENERAL_NEXT, true, 256, false, OUT_GENERAL>(),
 };
@@ -1792,7 +1793,7 @@ const Variant* pick_variant(int epi, bool rows, bool f4, bool tma, int64_t M, in
     double best_t = 0.0;
     for (const Variant& v : kVariants) {
         if (v.epi != epi || v.f4 != f4) continue;
-        if ((epi == EPI_LEAN || epi == EPI_NEXT) && v.rows != rows) continue;
+        if ((epi == EPI_LEAN || epi == EPI_NEXT || epi == EPI_RUNS) && v.rows != rows) continue;
         if (epi == EPI_LEAN && v.out == OUT_TMA && !tma) continue;
         const int64_t mt = (M + BM - 1) / BM, nt = (N + v.bn - 1) / v.bn;
         const int64_t slots = v.pair ? num_sms() / 2 : num_sms();
@@ -1980,7 +1981,7 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
                     : general ? (has_next ? EPI_GENERAL_NEXT : EPI_GENERAL)
                     : has_next ? EPI_NEXT
                     : sp.seg_group >= 0 ? EPI_SEG : EPI_LEAN;
-    const Variant* var = pick_variant(epi, a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0, a.M, a.N, (int)(sp.eb / KSTAGE));
+    const Variant* var = pick_variant(epi, runs ? a.acc_dbg != nullptr : a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0, a.M, a.N, (int)(sp.eb / KSTAGE));
     if (var == nullptr) return cudaErrorNotSupported;
     const int tile_n = var->bn;
     const bool pair = var->pair;
