@@ -181,13 +181,15 @@ namespace {
 
 cudaStream_t as_stream(soniq_stream_t s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// The staged path pays for its expansion passes and a persistent launch; below
-// about 2^30 multiply-adds the fused kernel is faster (measured: a 64 x 512 x
-// 512 layer 37 vs 17 us, decode M = 16 x 11008 x 4096 62 vs 41.5 us), unless
-// the call needs an epilogue only the staged kernel has.
+// With scratch, the staged path is the faster one where K is long (the fused kernel pays
+// about 4 us per 1024 codes) or the problem not tiny.  us, fused and staged: 64 x 512 x 512
+// 9.7, 7.7; 137 x 4096 x 1024 27.7, 15.6; 4000 x 256 x 128 10.8, 8.7; 3 x 3 convolutions
+// 1 x 56 x 56 x 64 14.9, 10.8 and 1 x 14 x 14 x 512 65, 24; 8000 x 128 x 128 9.7, 10.3.  (The
+// fused kernel also serves every call without scratch.)
 bool staged_worthwhile(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flags) {
     if (flags & SONIQ_FLAG_FORCE_STAGED) return true;
-    return (double)M * (double)N * (double)geo.K * (double)geo.taps >= 1073741824.0;
+    const int64_t K = (int64_t)geo.K * geo.taps;
+    return K >= 512 || (K >= 256 && (double)M * (double)N * (double)K >= 33554432.0);
 }
 
 // The kernel soniq_mp_gemm runs: a SONIQ_PATH_* value, -1 when the
