@@ -34,6 +34,8 @@
 // maxima found in a first pass over the rows, with a grid barrier.
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "soniq_device.cuh"
 #include "soniq_internal.h"
 #include "tc_ptx.cuh"
@@ -160,6 +162,11 @@ __device__ __forceinline__ void row_group_max(const uint8_t* row, const uint32_t
 
 namespace {
 
+// Per packed position: the channel's byte offset in a staged row, or in MODE 3,
+// whose kept tiles want the room, the channel in 16 bits.
+template <int MODE>
+using GatherOff = std::conditional_t<MODE == 3, uint16_t, uint32_t>;
+
 // Codes of nc <= 8 consecutive 32-code blocks of one group (positions pos0 +
 // 32 j of this lane) for rows rr0, rr0 + rgs, ... < nr of the tile, into the
 // code buffer.  Absent blocks of a short chunk read the zero slot and skip
@@ -173,12 +180,12 @@ namespace {
 // third of the stalls).  8192 x 4096 4/8 bits, given scales: 23.9 us before,
 // 22.3 now; 16384 x 3072 2/8 bits 56.5 and 41.
 template <int MODE>
-__device__ __forceinline__ void codes_chunk8(uint32_t rows_ba, uint32_t codes_a, const uint16_t* offs_s, int pos0, int nc,
+__device__ __forceinline__ void codes_chunk8(uint32_t rows_ba, uint32_t codes_a, const GatherOff<MODE>* offs_s, int pos0, int nc,
                                              int rr0, int rgs, int nr, uint32_t S, int npos, const GConst (*kc)[2],
                                              const GConst& kg, int g, float lv, uint32_t zero_slot) {
     uint32_t off[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) off[j] = j < nc ? 2u * offs_s[pos0 + 32 * j] : zero_slot;
+    for (int j = 0; j < 8; ++j) off[j] = j < nc ? (MODE == 3 ? 2u : 1u) * offs_s[pos0 + 32 * j] : zero_slot;
     uint32_t row = rows_ba + (uint32_t)rr0 * S, crow = codes_a + (uint32_t)(rr0 * npos + pos0);
     const float2 lv2 = make_float2(lv, lv);
 #pragma unroll 2
@@ -239,8 +246,8 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
     const int pa0 = p.g[0].pa, npos = pa0 + p.g[1].pa;
     const int c0 = p.g[0].count, c1 = p.g[1].count;
     // shared memory: channels | group masks (MODE 2: per channel; MODE 3: a bit each) | codes | staged rows
-    uint16_t* offs_s = reinterpret_cast<uint16_t*>(smem);
-    size_t o = ((size_t)npos * 2 + 15) & ~(size_t)15;
+    GatherOff<MODE>* offs_s = reinterpret_cast<GatherOff<MODE>*>(smem);
+    size_t o = ((size_t)npos * sizeof(GatherOff<MODE>) + 15) & ~(size_t)15;
     uint32_t* grp_s = reinterpret_cast<uint32_t*>(smem + o);
     if (MODE == 2) o += ((size_t)K * 2 + 15) & ~(size_t)15;
     if (MODE == 3) o += ((size_t)K / 8 + 19) & ~(size_t)15;
@@ -325,7 +332,7 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int q = q0 + u * nthr_c;
-            if (q < npos) offs_s[q] = (uint16_t)(ch[u] >= 0 ? ch[u] : K);   // padding: the zero slot
+            if (q < npos) offs_s[q] = (GatherOff<MODE>)((MODE == 3 ? 1 : 2) * (ch[u] >= 0 ? ch[u] : K));   // padding: the zero slot
             if (MODE >= 2 && q >= pa0 && ch[u] >= 0) {
                 if (MODE == 2) atomicOr(grp_s + (ch[u] >> 1), (ch[u] & 1) ? 0xFFFF0000u : 0x0000FFFFu);
                 else atomicOr(grp_s + (ch[u] >> 5), 1u << (ch[u] & 31));
@@ -554,7 +561,7 @@ bool gather_plan(const LayoutGeom& geo, int mode, int64_t M, const void* A, Gath
     }
     pl->rg = kGatherConsumerWarps / pl->wb;
     const size_t budget = kGatherSmemBudget;
-    const size_t fixed = (((size_t)pl->npos * 2 + 15) & ~(size_t)15) +
+    const size_t fixed = (((size_t)pl->npos * (mode == 3 ? 2 : 4) + 15) & ~(size_t)15) +
                          (mode == 2 ? (((size_t)geo.K * 2 + 15) & ~(size_t)15) : 0) +
                          (mode == 3 ? (((size_t)geo.K / 8 + 19) & ~(size_t)15) : 0) + 16;
     if (fixed >= budget) return false;

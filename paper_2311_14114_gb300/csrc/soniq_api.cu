@@ -375,16 +375,21 @@ soniq_status soniq_quantize_act(const soniq_layout* L, const void* A, int64_t M,
             // one pass: barrier words at the start of the scratch, per-CTA maxima after 256 bytes
             unsigned* bar = static_cast<unsigned*>(scratch);
             float* part = reinterpret_cast<float*>(static_cast<uint8_t*>(scratch) + 256);
-            // rows of 1 KB and more, two or more per SM, stream through the chip (8192 x 4096: 38.4 us,
-            // absmax pass + quantize pass 43.2; 16384 x 768: 21.6, one-pass kernel 24.2; 2048 x 4096: 16.4
-            // and 18.8); shorter rows are many small copies (12544 x 256: 15.4 and 11.6), fewer one row a CTA
-            cudaError_t e = cudaErrorNotSupported;
-            if (L->K >= 512 && M >= 2 * (int64_t)num_sms())
-                e = launch_quantize_stream(geo, L->perm, A16, M, s_a, Ap, s, bar, part, kMaxGridPartials,
-                                           kErrQuantBarrier);
+            // Large inputs stream through the chip (us: 8192 x 4096 38.4, absmax pass + quantize
+            // pass 43.2; 16384 x 768 21.6, one-pass kernel 24.2; 2048 x 4096 16.4, 18.8); smaller
+            // ones that fit on chip take the one-pass kernel (1500 x 1024 10.9, 9.9; 400 x 20000 24.3,
+            // 19.1; rows under 1 KB are many small copies: 12544 x 256 15.4, 11.6).
+            const bool streams = L->K >= 512 && M >= 2 * (int64_t)num_sms();
+            const bool large = M * (int64_t)L->K >= (6 << 20) && M >= 8 * (int64_t)num_sms();
+            auto stream = [&] {
+                return launch_quantize_stream(geo, L->perm, A16, M, s_a, Ap, s, bar, part, kMaxGridPartials,
+                                              kErrQuantBarrier);
+            };
+            cudaError_t e = streams && large ? stream() : cudaErrorNotSupported;
             if (e == cudaErrorNotSupported)
                 e = launch_quantize_fused(geo, L->perm, A16, M, s_a, Ap, s, bar, part, kMaxGridPartials,
                                           kErrQuantBarrier);
+            if (e == cudaErrorNotSupported && streams && !large) e = stream();
             if (e == cudaSuccess) return SONIQ_OK;
             if (e != cudaErrorNotSupported) return cuda_status(e);
         }

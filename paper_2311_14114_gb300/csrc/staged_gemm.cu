@@ -858,15 +858,17 @@ __device__ __forceinline__ uint32_t low_bytes(uint32_t b0, uint32_t b1, uint32_t
 }
 
 // Sec. 3 step 2 on a pair of fp16 outputs under a calibrated scale (Markstein
-// quotient, the top clip on the input, rounding by adding 1.5 * 2^23: the
-// codes are the low bytes of the results).
+// quotient, the top clip on the input, its last step saturated to [0, 1], rounding
+// by adding 1.5 * 2^23: the codes are the low bytes of the results).
 __device__ __forceinline__ void next_codes2(uint32_t h2, const QConst& k, uint32_t& c0, uint32_t& c1) {
     const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&h2));
-    const float x0 = fmin_keep_nan(f.x, k.s), x1 = fmin_keep_nan(f.y, k.s);
-    const float p0 = __fmul_rn(x0, k.r), p1 = __fmul_rn(x1, k.r);
-    const float q0 = __fmaf_rn(__fmaf_rn(-p0, k.s, x0), k.r, p0), q1 = __fmaf_rn(__fmaf_rn(-p1, k.s, x1), k.r, p1);
-    c0 = __float_as_uint(__fadd_rn(fmaxf(__fmul_rn(q0, k.levels), 0.0f), 12582912.0f));
-    c1 = __float_as_uint(__fadd_rn(fmaxf(__fmul_rn(q1, k.levels), 0.0f), 12582912.0f));
+    const float2 x = make_float2(fmin_keep_nan(f.x, k.s), fmin_keep_nan(f.y, k.s));
+    const float2 q0 = mul2(x, make_float2(k.r, k.r));
+    const float2 e = fma2(q0, make_float2(-k.s, -k.s), x);
+    const float2 q = make_float2(fma_sat(e.x, k.r, q0.x), fma_sat(e.y, k.r, q0.y));
+    const float2 u = add2(mul2(q, make_float2(k.levels, k.levels)), 12582912.0f);
+    c0 = __float_as_uint(u.x);
+    c1 = __float_as_uint(u.y);
 }
 
 // The next layer's packed codes from the warp's code bytes: cw[4 j + i] holds,
