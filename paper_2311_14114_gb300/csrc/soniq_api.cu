@@ -192,6 +192,16 @@ bool staged_worthwhile(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t fla
     return K >= 512 || (K >= 256 && (double)M * (double)N * (double)K >= 33554432.0);
 }
 
+// The scratch bytes a call may use.  Scratch off the 256-byte grid is an error where only
+// the staged path will do (forced, a layout variant) or from 2^30 multiply-adds on; smaller
+// calls run without it.
+size_t usable_scratch(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flags, const void* scratch, size_t bytes) {
+    if (scratch == nullptr) return 0;
+    const bool optional = !geo.variant && !(flags & SONIQ_FLAG_FORCE_STAGED) &&
+                          (double)M * (double)N * (double)geo.K * (double)geo.taps < 1073741824.0;
+    return optional && !aligned(scratch, 256) ? 0 : bytes;
+}
+
 // The kernel soniq_mp_gemm runs: a SONIQ_PATH_* value, -1 when the
 // tensor-core kernel would be chosen but cannot take the layout (mma_check
 // says why), -2 when the GEMV was forced but cannot take the shape.
@@ -457,7 +467,7 @@ soniq_status soniq_mp_gemm(const soniq_layout* L, const uint8_t* Ap, const float
     if (next != nullptr)
         flags = (flags & ~(uint32_t)(SONIQ_FLAG_FORCE_GEMV | SONIQ_FLAG_FORCE_SKINNY)) | SONIQ_FLAG_FORCE_MMA |
                 SONIQ_FLAG_FORCE_STAGED;
-    const int path = gemm_path(geo, M, N, flags, scratch != nullptr ? scratch_bytes : 0);
+    const int path = gemm_path(geo, M, N, flags, usable_scratch(geo, M, N, flags, scratch, scratch_bytes));
     if (next != nullptr && path != SONIQ_PATH_TENSOR_STAGED) return SONIQ_ERR_UNSUPPORTED;
     if (path < 0) return path == -2 ? SONIQ_ERR_UNSUPPORTED : mma_check(geo);
     if (path == SONIQ_PATH_GEMV || path == SONIQ_PATH_TENSOR_SKINNY) {
@@ -518,8 +528,9 @@ soniq_status soniq_mp_conv2d(const soniq_layout* L, const soniq_conv_desc* cd, c
     if (!aligned(Xp, 4) || !aligned(Wp, 16) || !aligned(Y, 16) || !aligned(s_a, 4) || !aligned(s_w, 4) ||
         (acc_dbg != nullptr && !aligned(acc_dbg, 4)))
         return SONIQ_ERR_ALIGNMENT;
-    const bool staged = !(flags & SONIQ_FLAG_FORCE_FUSED) && scratch != nullptr &&
-                        staged_worthwhile(geo, M, cd->C_out, flags) && staged_scratch_bytes(geo, M, cd->C_out) > 0 &&
+    scratch_bytes = usable_scratch(geo, M, cd->C_out, flags, scratch, scratch_bytes);
+    const bool staged = !(flags & SONIQ_FLAG_FORCE_FUSED) && staged_worthwhile(geo, M, cd->C_out, flags) &&
+                        staged_scratch_bytes(geo, M, cd->C_out) > 0 &&
                         (int64_t)scratch_bytes >= staged_scratch_bytes(geo, M, cd->C_out);
     if (staged && !aligned(scratch, 256)) return SONIQ_ERR_ALIGNMENT;
     if (next != nullptr && !staged) return SONIQ_ERR_UNSUPPORTED;
