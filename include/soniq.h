@@ -134,8 +134,8 @@ enum {
                                             scratch for the staged path is given */
     SONIQ_FLAG_FORCE_STAGED = 8u,        /* tensor-core work takes the staged path whenever the
                                             scratch suffices, however small the problem (without
-                                            it the staged path is used from K = 512 on, and from
-                                            K = 256 on for 2^25 multiply-adds and more) */
+                                            it the staged path is used from 2^30 multiply-adds
+                                            on, and for most smaller calls with long rows) */
     SONIQ_FLAG_FORCE_SKINNY = 16u,       /* tensor-core work takes the skinny swap-AB kernel
                                             (M <= 32, taps = 1, groups padded to 128 codes) */
     SONIQ_FLAG_TEST_DROP_ARRIVE = 0x100u /* test hook: the tensor-core kernels' operand producer

@@ -181,15 +181,25 @@ namespace {
 
 cudaStream_t as_stream(soniq_stream_t s) { return reinterpret_cast<cudaStream_t>(s); }
 
-// With scratch, the staged path is the faster one where K is long (the fused kernel pays
-// about 4 us per 1024 codes) or the problem not tiny.  us, fused and staged: 64 x 512 x 512
-// 9.7, 7.7; 137 x 4096 x 1024 27.7, 15.6; 4000 x 256 x 128 10.8, 8.7; 3 x 3 convolutions
-// 1 x 56 x 56 x 64 14.9, 10.8 and 1 x 14 x 14 x 512 65, 24; 8000 x 128 x 128 9.7, 10.3.  (The
-// fused kernel also serves every call without scratch.)
+// Whether scratch pays.  From 2^30 multiply-adds on the staged path is the rule; rows under
+// 256 codes (512 below 2^25 multiply-adds) stay on the fused kernel, which also serves every
+// call without scratch.  Between these the shorter of two estimates decides: the fused kernel
+// takes about 8 us per wave of its 128 x 128 tiles and 4 (a convolution 10) per 1024 codes of
+// it; the staged path about 8 us and 0.45 per MB of expanded operands.  us, fused and staged:
+// 64 x 512 x 512 (M, K, N) 9.7, 7.7; 137 x 4096 x 1024 27.7, 15.6; 100000 x 512 x 16 59.8, 39.7;
+// 4000 x 256 x 128 10.8, 8.7; 16000 x 1024 x 64 13.3, 14.9; 30000 x 1024 x 8 at 8 bits 27.7, 30.3;
+// 33 x 512 x 8192 10.1, 11.3; 3 x 3 convolutions 1 x 56 x 56 x 64 14.9, 10.8 and 1 x 14 x 14 x 512
+// 65, 24; 5 x 5, 64 x 28 x 28 x 64 -> 8, 68, 79.
 bool staged_worthwhile(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flags) {
     if (flags & SONIQ_FLAG_FORCE_STAGED) return true;
     const int64_t K = (int64_t)geo.K * geo.taps;
-    return K >= 512 || (K >= 256 && (double)M * (double)N * (double)K >= 33554432.0);
+    const double macs = (double)M * (double)N * (double)K;
+    if (macs >= 1073741824.0) return true;
+    if (K < 256 || (K < 512 && macs < 33554432.0)) return false;
+    const int64_t sms = num_sms() > 0 ? num_sms() : 152;
+    const int64_t waves = (((M + 127) / 128) * ((N + 127) / 128) + sms - 1) / sms;
+    const double fused_us = (double)waves * (8.0 + (geo.taps > 1 ? 10.0 : 4.0) * (double)K / 1024.0);
+    return 8.0 + 0.45e-6 * (double)staged_scratch_bytes(geo, M, N) < fused_us;
 }
 
 // The scratch bytes a call may use.  Scratch off the 256-byte grid is an error where only
