@@ -965,7 +965,8 @@ struct ColLoad {
     __device__ __forceinline__ void load(const SParams& p, const ColPlan<EPI>& cp, const FragTile& t, int epi_cols) {
         const int c = t.quad * (epi_cols / 4) + t.lane;
         const int n = t.nc0 + c < p.N ? t.nc0 + c : p.N - 1;
-        sw = __ldg(reinterpret_cast<const float2*>(p.s_w) + n);
+        // two scalar loads: s_w is 4-byte aligned, no more
+        sw = make_float2(__ldg(p.s_w + (int64_t)n * 2), __ldg(p.s_w + (int64_t)n * 2 + 1));
         cf = cp.centf ? __ldg(p.colsum + (int64_t)n * 2 + cp.gf) : 0;
         cl = cp.centl ? __ldg(p.colsum + (int64_t)n * 2 + cp.gl) : 0;
     }
