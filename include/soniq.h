@@ -265,18 +265,21 @@ SONIQ_API soniq_status soniq_pack_weights(const soniq_layout *layout, const floa
  *   scratch, scratch_bytes
  *              optional caller-owned device memory, 16-byte aligned.  With
  *              SONIQ_SCALE_PER_TENSOR and scratch_bytes >=
- *              soniq_quantize_act_scratch_bytes(), inputs whose rows fit on
- *              chip (about M * K <= 15 * 2^20) are quantized in one pass over
- *              A by a cooperative kernel whose grid barrier and per-CTA maxima
- *              live in the scratch; otherwise (or with scratch = NULL) the
- *              scale is found by a separate max-abs pass first.  Other modes
- *              ignore the scratch.
+ *              soniq_quantize_act_scratch_bytes(), one cooperative kernel whose
+ *              grid barrier and per-CTA maxima live in the scratch finds the
+ *              scale and forms the codes: in one pass over A where its rows fit
+ *              on chip (about M * K <= 15 * 2^20), or streaming the rows of a
+ *              large A twice.  With scratch = NULL, or where neither takes the
+ *              input, the scale is found by a separate max-abs pass first.
+ *              Inputs of at most 16384 values, other modes and the layout
+ *              variants ignore the scratch.
  *              Contract: the scratch must be zero-filled before its first use
  *              (cudaMemsetAsync once after allocating it); every completed
  *              call leaves it zero-filled again.  After soniq_sync_status
  *              reports SONIQ_ERR_TIMEOUT, zero it again before reuse.  Calls
  *              that may overlap on the GPU (different streams) must use
- *              different scratch buffers.
+ *              different scratch buffers; so must graphs that may be replayed
+ *              side by side, or beside direct calls.
  */
 SONIQ_API soniq_status soniq_quantize_act(const soniq_layout *layout, const void *A, int64_t M,
                                 int32_t scale_mode, float *s_a, uint8_t *Ap, void *scratch,

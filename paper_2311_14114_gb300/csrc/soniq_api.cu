@@ -242,6 +242,9 @@ int gemm_path(const LayoutGeom& geo, int64_t M, int32_t N, uint32_t flags, size_
     return SONIQ_PATH_TENSOR;
 }
 
+// A per-tensor input of at most this many values is quantized by one CTA where its rows fit.
+constexpr int64_t kOneCtaValues = 16384;
+
 // Checks a quantize-in-epilogue descriptor against this call's output width N.
 soniq_status check_next(const soniq_next_layer* next, int64_t N, int32_t out_dtype, LayoutGeom* geo_next) {
     if (next->layout == nullptr || next->s_a == nullptr || next->Ap == nullptr) return SONIQ_ERR_INVALID_ARG;
@@ -365,7 +368,10 @@ soniq_status soniq_pack_weights(const soniq_layout* L, const float* W, int32_t N
 int64_t soniq_quantize_act_scratch_bytes(const soniq_layout* L, int64_t M, int32_t scale_mode) {
     LayoutGeom geo;
     if (make_geom(L, 1, &geo) != SONIQ_OK || M < 0 || check_scale_mode_act(scale_mode) != SONIQ_OK) return -1;
-    return scale_mode == SONIQ_SCALE_PER_TENSOR && M > 0 ? kQuantScratchBytes : 0;
+    if (scale_mode != SONIQ_SCALE_PER_TENSOR || M == 0) return 0;
+    // none is read for the layout variants, nor by the one-CTA path, which takes 64 rows however
+    // the input is aligned
+    return geo.variant || (M <= 64 && M * (int64_t)L->K <= kOneCtaValues) ? 0 : kQuantScratchBytes;
 }
 
 soniq_status soniq_quantize_act(const soniq_layout* L, const void* A, int64_t M, int32_t scale_mode,
@@ -385,8 +391,8 @@ soniq_status soniq_quantize_act(const soniq_layout* L, const void* A, int64_t M,
     const uint16_t* A16 = static_cast<const uint16_t*>(A);
     if (geo.variant) return cuda_status(launch_variant_quantize_act(geo, L->perm, A16, M, scale_mode, s_a, Ap, s));
     if (scale_mode == SONIQ_SCALE_PER_TENSOR) {
-        // a small input (up to 16K values): one CTA finds the scale and quantizes, no scratch needed
-        if (M * (int64_t)L->K <= 16384) {
+        // a small input: one CTA finds the scale and quantizes, no scratch needed
+        if (M * (int64_t)L->K <= kOneCtaValues) {
             cudaError_t e0 = launch_quantize_rows(geo, L->perm, A16, M, scale_mode, true, s_a, Ap, s);
             if (e0 == cudaSuccess) return SONIQ_OK;
             if (e0 != cudaErrorNotSupported) return cuda_status(e0);

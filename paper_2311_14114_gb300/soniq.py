@@ -147,19 +147,20 @@ def _need(t: torch.Tensor, dtype, name: str):
 # barrier must start at zero and which every completed call leaves zeroed) is
 # never shared with the GEMM scratch (which the staged path overwrites).
 # Each is zero-filled when created and grows by reallocation when a call
-# needs more.  A GEMM call that is being captured takes its scratch from the
+# needs more.  A call that is being captured takes its scratch from the
 # graph's own memory instead: graphs that share a capture stream may be
-# replayed side by side, and a later, larger call may replace the cached buffer.
+# replayed side by side, a later, larger call may replace the cached buffer,
+# and a zero fill that is captured happens only when its graph is replayed.  For
+# the quantize scratch that fill is part of the graph (8.4 KB, one node).
 _scratch = {}
 
 
 def _get_scratch(nbytes: int, device, stream, use: str) -> Optional[torch.Tensor]:
     if nbytes <= 0:
         return None
-    if use == "gemm":
-        with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
-            if torch.cuda.is_current_stream_capturing():
-                return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
+        if torch.cuda.is_current_stream_capturing():
+            return (torch.zeros if use == "quantize" else torch.empty)(nbytes, dtype=torch.uint8, device=device)
     index = device.index
     key = (use, index, _current(index) if stream is None else stream.cuda_stream)
     buf = _scratch.get(key)
