@@ -8,9 +8,9 @@
 //   * scale runs along K: a group's packed positions are cut into runs of
 //     sub_k, each with its own max-abs scale (the fine scale groups of the
 //     evaluation setup); scale arrays are [rows or 1][2][nb].
-// Rows are staged whole in shared memory, eight at a time (variant_rows_kernel);
-// rows off the 16-byte grid, or too long for that, take two plain kernels that
-// read through the permutation from global memory.
+// Rows are staged whole in shared memory, several at a time (variant_rows_kernel);
+// rows too long for that, and a few long rows under given scales, take two plain
+// kernels that read through the permutation from global memory.
 #include <cuda_fp16.h>
 #include <stdint.h>
 
@@ -120,15 +120,23 @@ __global__ void __launch_bounds__(256) variant_codes_kernel(const T* X, int64_t 
 // ---- staged rows ---------------------------------------------------------------
 //
 // The plain kernels are bound by latency: a dependent global load per code, an
-// atomic per element for the maxima, a warp-wide OR per packed word (14 us for the
-// maxima and 24 us for the codes of a 1001 x 3000 fp16 input, 6 MB).  Here a CTA copies TR rows
-// with one bulk copy, and a warp takes a run (the positions that share a scale) in all of
-// them: lane = position within a 32-code block, so the permutation is read once per run;
-// a row's maximum is one warp reduction, nothing is synchronised across warps, and the
-// code bytes of the rows are packed a 32-code block per lane.
+// atomic per element for the maxima, a warp-wide OR per packed word.  Here a CTA copies a
+// tile of rows with one bulk copy, and a warp takes items of it: a chunk (four 32-code
+// blocks, which share a scale, since runs are multiples of 128 codes) in some of the rows.
+// Lane = position within a block, so the permutation is read once per item; a chunk's
+// maximum is one warp reduction, merged in shared memory; the code bytes are packed a
+// 32-code block per lane.  Items are chunks and not whole runs: a layout without runs has
+// one run per group, and one or two of the 16 warps would walk all of it.  Tiles hold no
+// more rows than give every SM two CTAs.  Signed 4/8 bits, per row, us with the plain
+// kernels, a warp per run in tiles of eight rows, and now: without runs 16 x 4096 9.2, 119,
+// 4.7; 8192 x 4096 347, 482, 67; weights 2048 x 4096 94, 243, 22; with 128-code runs
+// 1001 x 3000 37.7, 13.7, 10.8.  Now bound by the codes' IEEE divisions and, at few rows, by a
+// chain of an item's loads.
 constexpr int kVarWarps = 16;
-constexpr int kVarBlocks = 4;            // blocks of a run handled together
+constexpr int kVarBlocks = 4;            // blocks of a chunk
+constexpr int kVarRows = 8;              // rows of an item
 constexpr size_t kVarSmem = 200 * 1024;
+constexpr size_t kVarCodes = (size_t)kVarWarps * kVarRows * kVarBlocks * 32;   // the warps' code bytes
 enum { VAR_GIVEN = 0, VAR_ROW = 1, VAR_MAX = 2 };   // scales given; found per row; per-tensor maxima only
 
 template <typename T>
@@ -137,9 +145,27 @@ __device__ __forceinline__ float lds_x(const T* row, uint32_t c) {
     else return row[c];
 }
 
+// An item's place: chunk c of group g (run b), its channels ch (-1: padding).
+struct VItem {
+    int g, c, b, ch[kVarBlocks];
+    __device__ __forceinline__ VItem(const VGeo& v, const int32_t* perm, int chunk, int lane) {
+        const int nc0 = v.blocks[0] / kVarBlocks;
+        g = chunk >= nc0;
+        c = chunk - (g ? nc0 : 0);
+        b = v.sub_k > 0 ? c * (32 * kVarBlocks) / v.sub_k : 0;
+        const int count = g ? v.count1 : v.count0, base = g ? v.count0 : 0;
+#pragma unroll
+        for (int j = 0; j < kVarBlocks; ++j) {
+            const int pos = (c * kVarBlocks + j) * 32 + lane;
+            ch[j] = pos < count ? __ldg(perm + base + pos) : -1;
+        }
+    }
+};
+
+// tile_rows rows per CTA, of which every split-th belongs to an item.
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kVarWarps * 32) variant_rows_kernel(const T* X, int64_t rows, const int32_t* perm, VGeo v,
-                                                                     float* s, int per_row, int is_weight, int tile_rows,
+                                                                     float* s, int is_weight, int tile_rows, int split,
                                                                      uint8_t* out, unsigned* err, long long timeout_ns) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t bar_s;
@@ -147,25 +173,34 @@ __global__ void __launch_bounds__(kVarWarps * 32) variant_rows_kernel(const T* X
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t m0 = (int64_t)blockIdx.x * tile_rows;
     const int nr = rows - m0 < tile_rows ? (int)(rows - m0) : tile_rows;
+    const int nkeys = 2 * v.nb, items = (v.blocks[0] + v.blocks[1]) / kVarBlocks * split, nch = items / split;
     const uint32_t bar = tc::smem_u32(&bar_s), abort_flag = tc::smem_u32(&abort_s);
-    // code bytes [warp][tile row][4 blocks][32], then the rows
-    uint8_t* codes = smem + (size_t)warp * tile_rows * kVarBlocks * 32;
-    T* rows_s = reinterpret_cast<T*>(smem + (size_t)kVarWarps * tile_rows * kVarBlocks * 32);
+    // code bytes [warp][8 rows][4 blocks][32], the maxima [tile row][group][run] as bits, the rows
+    uint8_t* codes = smem + (size_t)warp * (kVarRows * kVarBlocks * 32);
+    uint32_t* max_s = reinterpret_cast<uint32_t*>(smem + kVarCodes);
+    uint8_t* stage = smem + kVarCodes + (MODE == VAR_GIVEN ? 0 : ((size_t)tile_rows * nkeys * 4 + 15) / 16 * 16);
     if (threadIdx.x == 0) {
         tc::mbar_init(bar, 1);
         tc::set_flag(abort_flag, 0);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (MODE != VAR_GIVEN)
+        for (int i = threadIdx.x; i < nr * nkeys; i += blockDim.x) max_s[i] = 0u;
     __syncthreads();
     tc::pdl_wait();      // launched with launch_pdl: every global access comes after this
+    // The tile keeps its global address modulo 16: one bulk copy of the aligned interior,
+    // plain loads of the few elements before and after it.
     const T* src = X + m0 * v.K;
-    const int64_t elems = (int64_t)nr * v.K;
-    const uint32_t bytes = (uint32_t)(elems * sizeof(T)), body = bytes & ~15u;
+    const uint32_t elems = (uint32_t)(nr * v.K);
+    const uint32_t head = min(elems, (uint32_t)((16u - ((uintptr_t)src & 15u)) & 15u) / (uint32_t)sizeof(T));
+    const uint32_t body = (elems - head) * (uint32_t)sizeof(T) & ~15u;
+    T* rows_s = reinterpret_cast<T*>(stage + ((uintptr_t)src & 15u));
     if (threadIdx.x == 0) {
         tc::mbar_arrive_expect_tx(bar, body);
-        if (body > 0) tc::bulk_load(tc::smem_u32(rows_s), src, body, bar);
+        if (body > 0) tc::bulk_load(tc::smem_u32(rows_s + head), src + head, body, bar);
     }
-    for (int64_t i = body / sizeof(T) + threadIdx.x; i < elems; i += blockDim.x) rows_s[i] = src[i];   // a last tile's end
+    if (threadIdx.x < head) rows_s[threadIdx.x] = src[threadIdx.x];
+    for (uint32_t i = head + body / (uint32_t)sizeof(T) + threadIdx.x; i < elems; i += blockDim.x) rows_s[i] = src[i];
     __syncthreads();
     if (!tc::wait_bounded_warp(bar, 0u, abort_flag, timeout_ns, err, kErrWait)) {
         // the copy in flight lands before the CTA exits
@@ -174,99 +209,102 @@ __global__ void __launch_bounds__(kVarWarps * 32) variant_rows_kernel(const T* X
             none_s = 0u;
             tc::wait_bounded(bar, 0u, tc::smem_u32(&none_s), timeout_ns, err, kErrWait);
         }
+        tc::set_flag(abort_flag, 1);
+    }
+
+    if (MODE != VAR_GIVEN) {
+        for (int it = warp; it < items; it += kVarWarps) {
+            const int part = it / nch;
+            const VItem w(v, perm, it - part * nch, lane);
+            const int key = w.g * v.nb + w.b;
+            for (int r = part; r < nr; r += split) {
+                float m = 0.0f;
+#pragma unroll
+                for (int j = 0; j < kVarBlocks; ++j)
+                    if (w.ch[j] >= 0) m = fmaxf(m, fabsf(lds_x<T>(rows_s + r * v.K, (uint32_t)w.ch[j])));   // skips NaN
+                // non-negative floats order as their bits
+                const uint32_t mb = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
+                if (lane == 0) atomicMax(max_s + r * nkeys + key, mb);
+            }
+        }
+    }
+    __syncthreads();
+    if (tc::abort_raised(abort_flag)) return;      // (a timed-out wait: nothing is written)
+    if (MODE == VAR_MAX) {
+        for (int key = threadIdx.x; key < nkeys; key += blockDim.x) {
+            uint32_t m = 0u;
+            for (int r = 0; r < nr; ++r) m = max(m, max_s[r * nkeys + key]);
+            if (m != 0u) atomicMax(reinterpret_cast<unsigned*>(s) + key, m);
+        }
         return;
     }
+    if (MODE == VAR_ROW)
+        for (int i = threadIdx.x; i < nr * nkeys; i += blockDim.x) s[m0 * nkeys + i] = __uint_as_float(max_s[i]);
 
-    // a warp per key (group, run): its blocks kb0 .. kb1 - 1 of the group
-    for (int key = warp; key < 2 * v.nb; key += kVarWarps) {
-        const int g = key >= v.nb, b = key - (g ? v.nb : 0);
-        const int rb = v.sub_k > 0 ? v.sub_k / 32 : v.blocks[g];
-        const int kb0 = b * rb, kb1 = min(v.blocks[g], kb0 + rb);
-        const int count = g ? v.count1 : v.count0, base = g ? v.count0 : 0;
-        const int n = v.bits[g], kind = v.kind[g];
+    for (int it = warp; it < items; it += kVarWarps) {
+        const int part = it / nch;
+        const VItem w(v, perm, it - part * nch, lane);
+        const int key = w.g * v.nb + w.b;
+        // (selects, not indexed loads: an indexed parameter array would live in local memory)
+        const int n = w.g ? v.bits[1] : v.bits[0], kind = w.g ? v.kind[1] : v.kind[0];
+        const int off = w.g ? v.off[1] : v.off[0];
         const float half = (float)(1 << (n - 1)), levels = (float)((1 << n) - 1);
         const uint32_t mask = (1u << n) - 1u;
-        // lane r: row r's scale
-        float sc = 0.0f;
-        if (MODE == VAR_GIVEN) {
-            if (lane < nr) sc = s[((per_row ? m0 + lane : 0) * 2 + g) * v.nb + b];
-        } else {
-            for (int k = kb0; k < kb1; k += kVarBlocks) {
-                int ch[kVarBlocks];
-#pragma unroll
-                for (int j = 0; j < kVarBlocks; ++j) {
-                    const int pos = (k + j) * 32 + lane;
-                    ch[j] = k + j < kb1 && pos < count ? __ldg(perm + base + pos) : -1;
-                }
-                for (int r = 0; r < nr; ++r) {
-                    float m = 0.0f;
-#pragma unroll
-                    for (int j = 0; j < kVarBlocks; ++j)
-                        if (ch[j] >= 0) m = fmaxf(m, fabsf(lds_x<T>(rows_s + (size_t)r * v.K, (uint32_t)ch[j])));   // skips NaN
-                    // non-negative floats order as their bits
-                    const uint32_t w = __reduce_max_sync(0xffffffffu, __float_as_uint(m));
-                    if (lane == r) sc = fmaxf(sc, __uint_as_float(w));
-                }
-            }
-            if (MODE == VAR_ROW && lane < nr) s[((m0 + lane) * 2 + g) * v.nb + b] = sc;
-            if (MODE == VAR_MAX) {
-                const uint32_t w = __reduce_max_sync(0xffffffffu, lane < nr ? __float_as_uint(sc) : 0u);
-                if (lane == 0 && w != 0u) atomicMax(reinterpret_cast<unsigned*>(s) + key, w);
-                continue;
-            }
-        }
-        for (int k = kb0; k < kb1; k += kVarBlocks) {
-            int ch[kVarBlocks];
+        float sc = MODE == VAR_GIVEN ? s[key] : 0.0f;
+        int k = 0;                                 // rows of the item
+        for (int r = part; r < nr; r += split, ++k) {
+            if (MODE == VAR_ROW) sc = __uint_as_float(max_s[r * nkeys + key]);
 #pragma unroll
             for (int j = 0; j < kVarBlocks; ++j) {
-                const int pos = (k + j) * 32 + lane;
-                ch[j] = k + j < kb1 && pos < count ? __ldg(perm + base + pos) : -1;
-            }
-            for (int r = 0; r < nr; ++r) {
-                const float sr = __shfl_sync(0xffffffffu, sc, r);
-#pragma unroll
-                for (int j = 0; j < kVarBlocks; ++j) {
-                    uint32_t pattern = 0u;
-                    if (ch[j] >= 0) {
-                        const float x = lds_x<T>(rows_s + (size_t)r * v.K, (uint32_t)ch[j]);
-                        if (kind == 2) pattern = x >= 0.0f ? 1u : 0u;
-                        else if (kind == 1 || is_weight) pattern = (uint32_t)weight_code(x, sr, half) & mask;
-                        else pattern = act_code(x, sr, levels);
-                    }
-                    codes[(r * kVarBlocks + j) * 32 + lane] = (uint8_t)pattern;
+                uint32_t pattern = 0u;
+                if (w.ch[j] >= 0) {
+                    const float x = lds_x<T>(rows_s + r * v.K, (uint32_t)w.ch[j]);
+                    if (kind == 2) pattern = x >= 0.0f ? 1u : 0u;
+                    else if (kind == 1 || is_weight) pattern = (uint32_t)weight_code(x, sc, half) & mask;
+                    else pattern = act_code(x, sc, levels);
                 }
+                codes[(k * kVarBlocks + j) * 32 + lane] = (uint8_t)pattern;
             }
-            __syncwarp();
-            // lane -> (row, block)
-            for (int i = lane; i < nr * kVarBlocks; i += 32) {
-                const int r = i / kVarBlocks, j = i % kVarBlocks;
-                if (k + j < kb1) {
-                    const uint4* c = reinterpret_cast<const uint4*>(codes + i * 32);
-                    const uint4 lo = c[0], hi = c[1];
-                    const uint32_t o[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-                    store_block32_n(n, o, out + (m0 + r) * v.row_bytes + v.off[g] + (int64_t)(k + j) * 4 * n);
-                }
-            }
-            __syncwarp();
         }
+        __syncwarp();
+        // lane -> (row, block)
+        if (lane < k * kVarBlocks) {
+            const int r = part + lane / kVarBlocks * split, j = lane % kVarBlocks;
+            const uint4* c = reinterpret_cast<const uint4*>(codes + lane * 32);
+            const uint4 lo = c[0], hi = c[1];
+            const uint32_t o[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+            store_block32_n(n, o, out + (m0 + r) * v.row_bytes + off + (int64_t)(w.c * kVarBlocks + j) * 4 * n);
+        }
+        __syncwarp();
     }
 }
+static_assert(kVarRows * kVarBlocks == 32, "an item's blocks are packed one per lane");
 
-// Rows per tile of variant_rows_kernel: the most of 8, 4, 2, 1 that fit and keep
-// tiles on the 16-byte grid; 0: none.
-template <typename T>
-int variant_tile_rows(const T* X, int32_t K, size_t* smem) {
-    for (int tr = 8; tr >= 1; tr /= 2) {
-        const size_t row_bytes = (size_t)K * sizeof(T);
-        *smem = (size_t)kVarWarps * tr * kVarBlocks * 32 + (size_t)tr * row_bytes;
-        if ((uintptr_t)X % 16 == 0 && (tr * row_bytes) % 16 == 0 && *smem <= kVarSmem) return tr;
-    }
-    return 0;
+// Rows per tile of variant_rows_kernel, the rows' split and the shared memory; false where
+// one row does not fit.
+bool variant_plan(const VGeo& v, int64_t rows, size_t elem, int* tile_rows, int* split, size_t* smem) {
+    const int nch = (v.blocks[0] + v.blocks[1]) / kVarBlocks;
+    const size_t row = (size_t)v.K * elem + 2 * v.nb * 4;
+    const size_t fixed = kVarCodes + 32;
+    if (fixed + row > kVarSmem || nch == 0) return false;
+    // rows of an item: up to eight; layouts with fewer chunks than warps split the tile's rows
+    *split = nch < kVarWarps ? kVarWarps / nch : 1;
+    int64_t tr = (int64_t)kVarRows * *split;
+    // two CTAs per SM where that leaves two rows each, and as many tiles as CTAs fit
+    const size_t half = kVarSmem / 2;
+    const int64_t fit = (int64_t)(((fixed + 2 * row <= half ? half : kVarSmem) - fixed) / row);
+    const int64_t ctas = 2 * (int64_t)num_sms(), share = (rows + ctas - 1) / ctas;
+    if (tr > fit) tr = fit;
+    if (tr > share) tr = share;
+    if (*split > tr) *split = (int)tr;
+    *tile_rows = (int)tr;
+    *smem = kVarCodes + ((size_t)tr * 2 * v.nb * 4 + 15) / 16 * 16 + (size_t)tr * v.K * elem + 16;
+    return (rows + tr - 1) / tr <= 2147483647;
 }
 
 template <typename T, int MODE>
-cudaError_t launch_variant_rows(const T* X, int64_t rows, const int32_t* perm, const VGeo& v, float* s, int per_row,
-                                int is_weight, int tile_rows, size_t smem, uint8_t* out, cudaStream_t st) {
+cudaError_t launch_variant_rows(const T* X, int64_t rows, const int32_t* perm, const VGeo& v, float* s, int is_weight,
+                                int tile_rows, int split, size_t smem, uint8_t* out, cudaStream_t st) {
     static bool attr_done[64] = {};
     int dev = 0;
     cudaGetDevice(&dev);
@@ -282,7 +320,7 @@ cudaError_t launch_variant_rows(const T* X, int64_t rows, const int32_t* perm, c
     if (err == nullptr) return cudaErrorUnknown;
     const int64_t tiles = (rows + tile_rows - 1) / tile_rows;
     const cudaError_t e = launch_pdl(variant_rows_kernel<T, MODE>, dim3((unsigned)tiles), dim3(kVarWarps * 32), smem, st, X,
-                                     rows, perm, v, s, per_row, is_weight, tile_rows, out, err, 2000000000LL);
+                                     rows, perm, v, s, is_weight, tile_rows, split, out, err, 2000000000LL);
     if (e == cudaSuccess) note_launch();
     return e;
 }
@@ -312,16 +350,19 @@ cudaError_t run_variant(const LayoutGeom& geo, const int32_t* perm, const T* X, 
     const int per_row = scale_mode == SONIQ_SCALE_PER_ROW;
     cudaError_t e = cudaSuccess;
     size_t smem = 0;
-    const int tr = variant_tile_rows(X, v.K, &smem);
-    if (tr > 0 && (rows + tr - 1) / tr <= 2147483647) {
-        if (per_row)
-            return launch_variant_rows<T, VAR_ROW>(X, rows, perm, v, s, 1, weight, tr, smem, out, st);
+    int tr = 0, split = 0;
+    // Given scales, few long rows: a tile of one row keeps 16 warps busy for K / 2048 items each,
+    // where the plain kernel spreads the row's blocks over the chip (signed 4/8 bits, us, plain and
+    // staged: 16 x 4096 2.6, 3.7; 64 x 4096 4.0, 3.6; 64 x 16384 9.2, 10.3; 256 x 4096 9.2, 4.5).
+    const bool plain = scale_mode == SONIQ_SCALE_CALIBRATED && rows <= 64 && v.K >= 2048;
+    if (!plain && variant_plan(v, rows, sizeof(T), &tr, &split, &smem)) {
+        if (per_row) return launch_variant_rows<T, VAR_ROW>(X, rows, perm, v, s, weight, tr, split, smem, out, st);
         if (scale_mode != SONIQ_SCALE_CALIBRATED) {
             if ((e = cudaMemsetAsync(s, 0, sizeof(float) * 2 * v.nb, st)) != cudaSuccess) return e;
-            if ((e = launch_variant_rows<T, VAR_MAX>(X, rows, perm, v, s, 0, weight, tr, smem, out, st)) != cudaSuccess)
+            if ((e = launch_variant_rows<T, VAR_MAX>(X, rows, perm, v, s, weight, tr, split, smem, out, st)) != cudaSuccess)
                 return e;
         }
-        return launch_variant_rows<T, VAR_GIVEN>(X, rows, perm, v, s, 0, weight, tr, smem, out, st);
+        return launch_variant_rows<T, VAR_GIVEN>(X, rows, perm, v, s, weight, tr, split, smem, out, st);
     }
     if (scale_mode != SONIQ_SCALE_CALIBRATED) {
         if (!per_row && (e = cudaMemsetAsync(s, 0, sizeof(float) * 2 * v.nb, st)) != cudaSuccess) return e;
