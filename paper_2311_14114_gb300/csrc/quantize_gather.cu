@@ -175,10 +175,9 @@ using GatherOff = std::conditional_t<MODE == 3, uint16_t, uint32_t>;
 //
 // Bound by instruction issue.  Two codes share each packed fp32 instruction,
 // and the clip at 0 (and of a NaN) is the saturation of the quotient's last
-// step: 6 instructions a code instead of 10.  The rows are a short loop: with
+// step: 6 instructions a code instead of 10.  The rows are a loop of one: with
 // all eight unrolled the kernel's instructions came cold for every tile (a
-// third of the stalls).  8192 x 4096 4/8 bits, given scales: 23.9 us before,
-// 22.3 now; 16384 x 3072 2/8 bits 56.5 and 41.
+// third of the stalls), with two 2048 x 16384 took 47 us instead of 42.
 template <int MODE>
 __device__ __forceinline__ void codes_chunk8(uint32_t rows_ba, uint32_t codes_a, const GatherOff<MODE>* offs_s, int pos0, int nc,
                                              int rr0, int rgs, int nr, uint32_t S, int npos, const GConst (*kc)[2],
@@ -188,7 +187,7 @@ __device__ __forceinline__ void codes_chunk8(uint32_t rows_ba, uint32_t codes_a,
     for (int j = 0; j < 8; ++j) off[j] = j < nc ? (MODE == 3 ? 2u : 1u) * offs_s[pos0 + 32 * j] : zero_slot;
     uint32_t row = rows_ba + (uint32_t)rr0 * S, crow = codes_a + (uint32_t)(rr0 * npos + pos0);
     const float2 lv2 = make_float2(lv, lv);
-#pragma unroll 2
+#pragma unroll 1
     for (int r = rr0; r < nr; r += rgs, row += (uint32_t)rgs * S, crow += (uint32_t)(rgs * npos)) {
         const GConst kk = MODE == 2 ? kc[r][g] : kg;
         if (kk.mode == 1) {
@@ -318,7 +317,9 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
         for (int w = tid; w < words; w += nthr_c) grp_s[w] = 0u;
         consumer_sync();
     }
-    // channels: the permutation's loads issued eight at a time
+    // channels: the permutation's loads issued eight at a time.  The offsets are stored in a
+    // loop of their own, the masks marked in another: with both in one loop given scales took
+    // 11.1 us for 1 x 16384 (6.9 so), 7.8 for 400 x 8192 (5.5), 21.3 for 8192 x 4096 (19.0).
     for (int q0 = tid; q0 < npos; q0 += 8 * nthr_c) {
         int ch[8];
 #pragma unroll
@@ -332,8 +333,15 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
 #pragma unroll
         for (int u = 0; u < 8; ++u) {
             const int q = q0 + u * nthr_c;
-            if (q < npos) offs_s[q] = (GatherOff<MODE>)((MODE == 3 ? 1 : 2) * (ch[u] >= 0 ? ch[u] : K));   // padding: the zero slot
-            if (MODE >= 2 && q >= pa0 && ch[u] >= 0) {
+            // padding: the zero slot
+            if (q < npos)
+                offs_s[q] = (GatherOff<MODE>)(MODE == 3 ? (ch[u] >= 0 ? ch[u] : K)
+                                                        : (ch[u] >= 0 ? 2u * (uint32_t)ch[u] : row_bytes));
+        }
+        if constexpr (MODE >= 2) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                if (q0 + u * nthr_c < pa0 || ch[u] < 0) continue;
                 if (MODE == 2) atomicOr(grp_s + (ch[u] >> 1), (ch[u] & 1) ? 0xFFFF0000u : 0x0000FFFFu);
                 else atomicOr(grp_s + (ch[u] >> 5), 1u << (ch[u] & 31));
             }
