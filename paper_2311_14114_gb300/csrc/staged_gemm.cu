@@ -56,6 +56,7 @@
 #include <cuda_fp16.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "packed_words.cuh"
 #include "soniq_device.cuh"
@@ -264,7 +265,7 @@ constexpr int kExpandRows = 4;      // rows a warp expands together
 // 32-byte sector in two instructions.  Four rows keep that many independent
 // loads in flight and share the index arithmetic.  Convolutions (64 x 56 x 56 x 64, 3 x 3,
 // 282 MB of operands: 192 us a call with one row per warp, 155 with four; 64 x 14 x 14 x 256
-// 29.7 and 29.2) and rows that expand_stream_kernel does not take.
+// 29.7 and 29.2; their weights' rows in the same launch).
 template <int N, int PARTS>
 __device__ __forceinline__ void expand_rows(const ExpandParams& p, int64_t r0, int g, int lane) {
     using Words = PartWords<N, PARTS>;
@@ -387,10 +388,14 @@ __global__ void __launch_bounds__(256, 4) expand_kernel(const __grid_constant__ 
 // once per 32 pieces, and the short kernel's straight-line code is fetched
 // cold: 20 us for the 8192 x 4096 x 4096 4/8-bit layer (94 MB moved), most stalls on
 // loads and on instruction fetch; streamed, 13 us.  Here a producer warp
-// streams tiles of eight packed rows (contiguous, so one bulk copy each)
+// streams tiles of packed rows (contiguous, so one bulk copy each)
 // through a ring; each consumer warp expands one row of a tile, two pieces per
 // step, with a short loop per group, and stores 512 contiguous bytes at a time.
-constexpr int kStreamWarps = 8;             // consumers: one row of a tile each
+// Rows of which eight do not fit twice are shared by two, four or eight warps, whose
+// code sums meet in shared memory; the producer writes them out when it takes the
+// stage back (8 bits, calls in us, from global memory and streamed: 1000 x 60000 x 64
+// 457, 259; 137 x 11008 x 11008 173, 128; 4096 x 7000 x 1024 86, 69).
+constexpr int kStreamWarps = 8;             // consumers
 constexpr int kStreamMaxStages = 6;
 constexpr size_t kStreamSmemPerSm = 216 * 1024;
 
@@ -399,11 +404,15 @@ struct StreamParams {
     unsigned* err;
     int32_t stages, stage_bytes;
     int32_t rpw;              // rows of a tile per warp
+    int32_t wpr;              // warps per row (1, 2, 4 or 8; rpw is 1 above 1)
 };
 
-// One group of nr staged rows (row r's packed codes at src), by one warp.
+// One group of nr staged rows (row r's packed codes at src), by one warp of wpr: its
+// pieces are those of index sub modulo wpr, 32 at a time.  sum: wpr > 1, the shared
+// word of the row's and group's code sum.
 template <int N, int PARTS>
-__device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src, int64_t r, int nr, int g, int lane) {
+__device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src, int64_t r, int nr, int g, int lane, int sub,
+                                             int wpr, int32_t* sum) {
     const bool vec8 = p.vec8[g] != 0;
     const int ck = p.code_kind[g];
     const __half2 bias = __half2half2(__ushort_as_half(
@@ -414,7 +423,7 @@ __device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src
     for (int i = 0; i < nr; ++i, src += (uint32_t)p.src_row_bytes, drow += p.dst_row_bytes) {
         int32_t csum = 0;
 #pragma unroll 2
-        for (int c = lane; c < pieces; c += 32) {
+        for (int c = lane + 32 * sub; c < pieces; c += 32 * wpr) {
             const int kb = c / PARTS, part = c % PARTS;
             PartWords<N, PARTS> w;
             if (c < have) w.load(SharedWords{src + (uint32_t)(kb * 4 * N)}, part, vec8);
@@ -423,7 +432,10 @@ __device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src
         }
         if (PARTS == 4 && p.is_weight) {
             const int32_t s = __reduce_add_sync(0xffffffffu, csum);
-            if (lane == 0) p.colsum[(r + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
+            if (lane == 0) {
+                if (wpr == 1) p.colsum[(r + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
+                else atomicAdd(sum, s);
+            }
         }
     }
 }
@@ -432,6 +444,7 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full_bar[kStreamMaxStages], empty_bar[kStreamMaxStages];
     __shared__ uint32_t abort_s, none_s;
+    __shared__ int32_t sums_s[kStreamMaxStages][kStreamWarps];    // code sums [row of the tile][group], wpr > 1
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t abort_flag = tc::smem_u32(&abort_s), base = tc::smem_u32(smem);
     if (threadIdx.x == 0) {
@@ -443,38 +456,53 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
         none_s = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    if (threadIdx.x < kStreamMaxStages * kStreamWarps) (&sums_s[0][0])[threadIdx.x] = 0;
     __syncthreads();
     tc::pdl_wait();      // launched with launch_pdl: the packed rows are written before this
     // (no early trigger: GEMM CTAs that move in as this kernel's leave cost the MLP block 14 us)
-    const int tr = kStreamWarps * sp.rpw;                  // rows per tile
+    const int tr = kStreamWarps / sp.wpr * sp.rpw;         // rows per tile
     const int64_t tiles_a = (sp.op[0].rows + tr - 1) / tr;
     const int64_t tiles = tiles_a + (sp.op[1].rows + tr - 1) / tr;
     int b = 0;
     uint32_t ph = 0u;
     if (warp == kStreamWarps) {
         // ---- producer ----
+        // writes out the code sums of weight tile t, in stage st, and clears them
+        auto flush = [&](int64_t t, int st) {
+            const ExpandParams& p = sp.op[1];
+            const int64_t r = (t - tiles_a) * tr + (lane >> 1);
+            const int g = lane & 1;
+            if (t >= tiles_a && lane < 2 * tr && r < p.rows && p.kind[g] == 1 && p.blk_dst[g] > 0) {
+                p.colsum[r * 2 + g] = sums_s[st][lane] - (1 << (p.bits[g] - 1)) * 32 * p.blk_dst[g];
+                sums_s[st][lane] = 0;
+            }
+        };
+        const int64_t behind = (int64_t)sp.stages * gridDim.x;
         bool ok = true;
         int64_t issued = 0;
         for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x, ++issued) {
             if (issued >= sp.stages) {
                 ok = tc::wait_bounded_warp(tc::smem_u32(&empty_bar[b]), ph ^ 1u, abort_flag, kTimeoutNs, sp.err, kErrWait);
                 if (!ok) break;
+                if (sp.wpr > 1) flush(t - behind, b);
             }
             const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
             const int64_t r0 = (t < tiles_a ? t : t - tiles_a) * tr;
             const int nr = (int)(p.rows - r0 < tr ? p.rows - r0 : tr);
-            const int bytes = nr * (int)p.src_row_bytes, body = bytes & ~15;
-            const uint8_t* src = p.src + r0 * p.src_row_bytes;      // 16-byte aligned: eight rows of 4-byte multiples
-            const uint32_t dst = base + (uint32_t)(b * sp.stage_bytes), bar = tc::smem_u32(&full_bar[b]);
+            // the tile keeps its global address modulo 16: one bulk copy of the aligned interior,
+            // lanes 0..2 move the words before it, 4..6 those after it
+            const uint8_t* src = p.src + r0 * p.src_row_bytes;
+            const int shift = (int)((uintptr_t)src & 15u), bytes = nr * (int)p.src_row_bytes;
+            const int head = min((16 - shift) & 15, bytes), body = (bytes - head) & ~15, tail = bytes - head - body;
+            const uint32_t dst = base + (uint32_t)(b * sp.stage_bytes + shift), bar = tc::smem_u32(&full_bar[b]);
             if (lane == 0 && body > 0) {
                 asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(body)
                              : "memory");
-                tc::bulk_load(dst, src, (uint32_t)body, bar);
+                tc::bulk_load(dst + head, src + head, (uint32_t)body, bar);
             }
-            // a last tile may end within 16 bytes
-            if (lane < (bytes - body) / 4)
-                asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + body + 4 * lane),
-                             "r"(__ldg(reinterpret_cast<const uint32_t*>(src + body) + lane))
+            const int at = lane < 4 ? 4 * lane : head + body + 4 * (lane - 4);
+            if (lane < 4 ? 4 * lane < head : 4 * (lane - 4) < tail)
+                asm volatile("st.shared.u32 [%0], %1;" ::"r"(dst + at), "r"(__ldg(reinterpret_cast<const uint32_t*>(src + at)))
                              : "memory");
             __syncwarp();
             if (lane == 0) tc::mbar_arrive(bar);
@@ -483,47 +511,66 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
                 ph ^= 1u;
             }
         }
-        // abandoned: the copies in flight land before the CTA exits
-        if (!ok && lane == 0)
-            for (int i = 0; i < sp.stages; ++i)
-                tc::wait_bounded(tc::smem_u32(&full_bar[i]), i < b ? ph : ph ^ 1u, tc::smem_u32(&none_s), kTimeoutNs,
-                                 sp.err, kErrWait);
+        if (ok && sp.wpr > 1) {
+            // the code sums still in the ring
+            for (int64_t i = issued > sp.stages ? issued - sp.stages : 0; i < issued && ok; ++i) {
+                const int st = (int)(i % sp.stages);
+                ok = tc::wait_bounded_warp(tc::smem_u32(&empty_bar[st]), (uint32_t)(i / sp.stages) & 1u, abort_flag,
+                                           kTimeoutNs, sp.err, kErrWait);
+                if (ok) flush(blockIdx.x + i * gridDim.x, st);
+            }
+        }
+        // the copies in flight land before the CTA exits, also when it was abandoned
+        if (lane == 0)
+            for (int64_t i = issued > sp.stages ? issued - sp.stages : 0; i < issued; ++i)
+                tc::wait_bounded(tc::smem_u32(&full_bar[i % sp.stages]), (uint32_t)(i / sp.stages) & 1u, tc::smem_u32(&none_s),
+                                 kTimeoutNs, sp.err, kErrWait);
         return;
     }
-    // ---- consumers ----
+    // ---- consumers: warp -> rows row0 .. row0 + rpw - 1 of a tile, pieces sub modulo wpr ----
+    const int row0 = warp / sp.wpr * sp.rpw, sub = warp % sp.wpr;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         if (!tc::wait_bounded_warp(tc::smem_u32(&full_bar[b]), ph, abort_flag, kTimeoutNs, sp.err, kErrWait)) return;
         const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
-        const int64_t r = (t < tiles_a ? t : t - tiles_a) * tr + warp * sp.rpw;
+        const int64_t r0 = (t < tiles_a ? t : t - tiles_a) * tr, r = r0 + row0;
         const int nr = p.rows - r < sp.rpw ? (int)(p.rows - r) : sp.rpw;
         if (nr > 0) {
-            uint32_t row = base + (uint32_t)(b * sp.stage_bytes) + (uint32_t)(warp * sp.rpw * (int)p.src_row_bytes);
+            uint32_t row = base + (uint32_t)(b * sp.stage_bytes) + ((uint32_t)(uintptr_t)(p.src + r0 * p.src_row_bytes) & 15u) +
+                           (uint32_t)(row0 * (int)p.src_row_bytes);
             asm volatile("" : "+r"(row)::"memory");        // keeps the row's loads behind the wait
 #pragma unroll 1
             for (int g = 0; g < 2; ++g) {
                 if (p.blk_dst[g] == 0) continue;
                 const uint32_t src = row + (uint32_t)p.src_off[g];
                 const int n = p.bits[g];
+                int32_t* sum = &sums_s[b][2 * (warp / sp.wpr) % kStreamWarps + g];
+                auto group = [&](auto bits, auto parts) {
+                    stream_group<decltype(bits)::value, decltype(parts)::value>(p, src, r, nr, g, lane, sub, sp.wpr, sum);
+                };
+                using std::integral_constant;
+                constexpr integral_constant<int, 1> c1{};
+                constexpr integral_constant<int, 2> c2{};
+                constexpr integral_constant<int, 4> c4{};
                 if (p.kind[g] == 2) {
-                    if (n == 1) stream_group<1, 1>(p, src, r, nr, g, lane);
-                    else stream_group<2, 1>(p, src, r, nr, g, lane);
+                    if (n == 1) group(c1, c1);
+                    else group(c2, c1);
                 } else if (p.kind[g] == 0) {
                     switch (n) {
-                        case 1: stream_group<1, 2>(p, src, r, nr, g, lane); break;
-                        case 2: stream_group<2, 2>(p, src, r, nr, g, lane); break;
-                        case 3: stream_group<3, 2>(p, src, r, nr, g, lane); break;
-                        default: stream_group<4, 2>(p, src, r, nr, g, lane); break;
+                        case 1: group(c1, c2); break;
+                        case 2: group(c2, c2); break;
+                        case 3: group(integral_constant<int, 3>{}, c2); break;
+                        default: group(c4, c2); break;
                     }
                 } else {
                     switch (n) {
-                        case 1: stream_group<1, 4>(p, src, r, nr, g, lane); break;
-                        case 2: stream_group<2, 4>(p, src, r, nr, g, lane); break;
-                        case 3: stream_group<3, 4>(p, src, r, nr, g, lane); break;
-                        case 4: stream_group<4, 4>(p, src, r, nr, g, lane); break;
-                        case 5: stream_group<5, 4>(p, src, r, nr, g, lane); break;
-                        case 6: stream_group<6, 4>(p, src, r, nr, g, lane); break;
-                        case 7: stream_group<7, 4>(p, src, r, nr, g, lane); break;
-                        default: stream_group<8, 4>(p, src, r, nr, g, lane); break;
+                        case 1: group(c1, c4); break;
+                        case 2: group(c2, c4); break;
+                        case 3: group(integral_constant<int, 3>{}, c4); break;
+                        case 4: group(c4, c4); break;
+                        case 5: group(integral_constant<int, 5>{}, c4); break;
+                        case 6: group(integral_constant<int, 6>{}, c4); break;
+                        case 7: group(integral_constant<int, 7>{}, c4); break;
+                        default: group(integral_constant<int, 8>{}, c4); break;
                     }
                 }
             }
@@ -537,14 +584,18 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
     }
 }
 
-// expand_stream_kernel where its ring takes the rows; false where it does not
-// (convolutions gather their rows; packed rows off the 16-byte grid or too long).
+// expand_stream_kernel for linear layers; false for convolutions, which gather their rows.
 bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st, cudaError_t* err) {
-    if (a.conv || (uintptr_t)a.src % 16 != 0 || (uintptr_t)w.src % 16 != 0) return false;
+    if (a.conv) return false;
     const int64_t row = a.src_row_bytes > w.src_row_bytes ? a.src_row_bytes : w.src_row_bytes;
     // four CTAs per SM, or two where four rings of two stages do not fit (rows over 3.4 KB;
-    // 8192 x 4096 x 4096 4/8 bits: two 101, three 99.7, four 99.4 us a call; 2/8 bits 81, 80, 79.6)
+    // 8192 x 4096 x 4096 4/8 bits: two 101, three 99.7, four 99.4 us a call; 2/8 bits 81, 80, 79.6),
+    // and then as few warps per row as two stages allow (two from 6.9 KB on, four, eight; the
+    // longest row, 64 KB, has one CTA per SM)
     int per_sm = kStreamWarps * row * 2 + 256 <= (int64_t)kStreamSmemPerSm / 4 ? 4 : 2;
+    int64_t wpr = 1;
+    while (wpr < kStreamWarps && kStreamWarps / wpr * row * 2 + 288 > (int64_t)kStreamSmemPerSm / per_sm) wpr *= 2;
+    if (kStreamWarps / wpr * row * 2 + 288 > (int64_t)kStreamSmemPerSm / per_sm) per_sm = 1;
     const int64_t smem_cta = (int64_t)kStreamSmemPerSm / per_sm;
     // short rows: several per warp and stage (about 12 KB), as long as every CTA gets two tiles
     // (16384 x 768 x 3072: 61 us a call, one row per warp 70)
@@ -552,9 +603,12 @@ bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st
     int64_t rpw = 12 * 1024 / (kStreamWarps * row);
     if (rpw > all / (2 * cap * kStreamWarps)) rpw = all / (2 * cap * kStreamWarps);
     if (rpw > 4) rpw = 4;
-    if (rpw < 1) rpw = 1;
-    const int64_t tr = kStreamWarps * rpw;
-    const int64_t stage = (tr * row + 127) / 128 * 128;
+    if (rpw < 1 || wpr > 1) rpw = 1;
+    const int64_t tr = kStreamWarps / wpr * rpw;
+    // (room to keep a tile's address modulo 16 where tiles do not start on that grid)
+    const bool grid16 = ((uintptr_t)a.src | (uintptr_t)w.src | (uintptr_t)(tr * a.src_row_bytes) |
+                         (uintptr_t)(tr * w.src_row_bytes)) % 16 == 0;
+    const int64_t stage = (tr * row + (grid16 ? 0 : 16) + 127) / 128 * 128;
     const int64_t stages = smem_cta / stage;
     if (stages < 2) return false;
     StreamParams sp;
@@ -565,6 +619,7 @@ bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st
     sp.stages = (int32_t)(stages < kStreamMaxStages ? stages : kStreamMaxStages);
     sp.stage_bytes = (int32_t)stage;
     sp.rpw = (int32_t)rpw;
+    sp.wpr = (int32_t)wpr;
     const int64_t tiles = (a.rows + tr - 1) / tr + (w.rows + tr - 1) / tr;
     static bool attr_done[64] = {};
     int dev = 0;
@@ -572,7 +627,7 @@ bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st
     if (dev < 0 || dev >= 64) return false;
     if (!attr_done[dev]) {
         *err = cudaFuncSetAttribute(expand_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kStreamSmemPerSm / 2);
+                                    (int)kStreamSmemPerSm);
         if (*err == cudaSuccess) *err = prefer_max_shared((const void*)expand_stream_kernel);
         if (*err != cudaSuccess) return true;
         attr_done[dev] = true;
