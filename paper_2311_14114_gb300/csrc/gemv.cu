@@ -348,7 +348,10 @@ __global__ void __launch_bounds__(bulk_threads<MT>(), 1) gemv_bulk_kernel(const 
 #pragma unroll
             for (int g = 0; g < 2; ++g) {
                 const GroupGeom& G = p.g[g];
-                if (G.pa == 0) continue;
+                if (G.pa == 0) {
+                    if (p.acc_dbg != nullptr) p.acc_dbg[((int64_t)g * p.M + m) * p.N + n] = 0;
+                    continue;
+                }
                 const uint32_t v = acc_s[(g * MT + m) * round_rows + rr];
                 const int32_t off = 1 << (G.bits_w - 1);
                 const int32_t a = (int32_t)(v - (uint32_t)(off * rowsum[g * 16 + m]));

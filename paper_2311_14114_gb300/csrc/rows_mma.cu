@@ -268,13 +268,13 @@ __global__ void __launch_bounds__(kRowsThreads, 1) rows_mma_kernel(const RowsPar
 #pragma unroll
         for (int g = 0; g < 2; ++g) {
             const GroupGeom& G = p.g[g];
-            if (G.pa == 0) continue;
             const int32_t a = acc_s[(g * p.M + m) * p.rows_pad + rr];
+            if (p.acc_dbg != nullptr) p.acc_dbg[((int64_t)g * p.M + m) * p.N + n0 + rr] = a;
+            if (G.pa == 0) continue;
             const float inv = 1.0f / ((float)((1 << G.bits_a) - 1) * (float)(1 << (G.bits_w - 1)));
             const float sw = sw_s[rr * 2 + g] * inv;
             const float sa = p.s_a_per_row ? __ldg(p.s_a + m * 2 + g) : __ldg(p.s_a + g);
             y = g == 0 ? (sa * sw) * (float)a : fmaf(sa * sw, (float)a, y);
-            if (p.acc_dbg != nullptr) p.acc_dbg[((int64_t)g * p.M + m) * p.N + n0 + rr] = a;
         }
         const int64_t idx = (int64_t)m * p.N + n0 + rr;
         if (p.out_bf16) reinterpret_cast<__nv_bfloat16*>(p.Y)[idx] = __float2bfloat16_rn(y);
