@@ -128,7 +128,7 @@ enum {
 enum { SONIQ_OUT_F16 = 0, SONIQ_OUT_BF16 = 1 };
 
 enum {
-    SONIQ_FLAG_FORCE_GEMV = 1u,          /* soniq_mp_gemm: use the GEMV for any M <= 16 */
+    SONIQ_FLAG_FORCE_GEMV = 1u,          /* soniq_mp_gemm: use the CUDA-core GEMV for any M <= 16 */
     SONIQ_FLAG_FORCE_MMA = 2u,           /* soniq_mp_gemm: use a tensor-core kernel for any M */
     SONIQ_FLAG_FORCE_FUSED = 4u,         /* tensor-core work takes the fused kernel even when
                                             scratch for the staged path is given */
@@ -140,22 +140,32 @@ enum {
                                             (M <= 32, taps = 1, groups padded to 128 codes) */
     SONIQ_FLAG_TEST_DROP_ARRIVE = 0x100u /* test hook: the tensor-core kernels' operand producer
                                             skips its first arrival (fused) or its first K-stage
-                                            (staged, skinny), so the consumer's bounded wait runs
+                                            (staged, skinny; the rows kernel from M = 13 on its
+                                            first weight rows), so the consumer's bounded wait runs
                                             out and the call reports SONIQ_ERR_TIMEOUT */
 };
 
-/* Kernels behind soniq_mp_gemm (see soniq_mp_gemm_path). */
+/* Paths of soniq_mp_gemm (see soniq_mp_gemm_path). */
 enum {
-    SONIQ_PATH_GEMV = 0,           /* GEMV streaming the packed weights (small M): dot products on CUDA
-                                      cores, or warp-level tensor instructions for M >= 3 */
+    SONIQ_PATH_GEMV = 0,           /* M <= SONIQ_GEMV_MAX_M, or forced (M <= 16): packed weights
+                                      streamed, no scratch */
     SONIQ_PATH_TENSOR = 1,         /* tcgen05 kernel expanding packed tiles on chip (no scratch) */
     SONIQ_PATH_TENSOR_STAGED = 2,  /* codes expanded once into scratch, then a tcgen05 GEMM */
-    SONIQ_PATH_TENSOR_SKINNY = 3   /* few rows, packed weight rows converted on chip: warp-level
-                                      tensor instructions where the activation rows fit in shared
-                                      memory, else a swap-AB tcgen05 kernel */
+    SONIQ_PATH_TENSOR_SKINNY = 3   /* M <= SONIQ_SKINNY_MAX_M: packed weight rows converted on
+                                      chip, no scratch */
 };
-/* Without flags, soniq_mp_gemm runs the GEMV for M <= SONIQ_GEMV_MAX_M and the
- * skinny tensor-core kernel for M <= SONIQ_SKINNY_MAX_M. */
+/* Kernels behind them (see soniq_mp_gemm_kernel). */
+enum {
+    SONIQ_KERNEL_GEMV = 0,         /* dot products on CUDA cores */
+    SONIQ_KERNEL_FUSED = 1,
+    SONIQ_KERNEL_STAGED = 2,
+    SONIQ_KERNEL_SKINNY = 3,       /* swap-AB tcgen05 kernel */
+    SONIQ_KERNEL_ROWS = 4          /* warp-level tensor instructions: the GEMV and skinny paths from
+                                      M = 3 on, where the activation rows fit in shared memory
+                                      and no flag forces one of the two kernels above */
+};
+/* Without flags, soniq_mp_gemm takes the GEMV path for M <= SONIQ_GEMV_MAX_M and the
+ * skinny path for M <= SONIQ_SKINNY_MAX_M. */
 #define SONIQ_GEMV_MAX_M 12
 #define SONIQ_SKINNY_MAX_M 32
 
@@ -334,10 +344,10 @@ SONIQ_API soniq_status soniq_quantize_act_oneshot(const soniq_layout *layout, co
  *   Acc_g[m][n] = sum over k in group g of u[m][k] * j[n][k]   (exact int32)
  *   Y[m][n]     = sum_g s_a(m,g) * s_w[n][g] / ((2^na_g - 1) * 2^(nw_g - 1)) * Acc_g[m][n]
  * computed in fp32 and rounded to nearest fp16 (or bf16).  M <= SONIQ_GEMV_MAX_M
- * runs a GEMV over the packed weights, M <= SONIQ_SKINNY_MAX_M a skinny
- * tensor-core kernel, larger M the tcgen05 GEMM (flags can force a
+ * takes the GEMV path over the packed weights, M <= SONIQ_SKINNY_MAX_M the skinny
+ * path, larger M the tcgen05 GEMM (flags can force a
  * kernel; the GEMV takes M <= 16, the skinny kernel M <= 32);
- * soniq_mp_gemm_path tells which.
+ * soniq_mp_gemm_path tells the path, soniq_mp_gemm_kernel the kernel.
  *
  *   Ap, s_a    from soniq_quantize_act with the same layout (pad_unit 32 or 128);
  *              s_a [2] (PER_TENSOR / CALIBRATED) or [M][2] (PER_ROW).
@@ -371,10 +381,14 @@ SONIQ_API soniq_status soniq_mp_gemm(const soniq_layout *layout, const uint8_t *
  * bits.  The scratch needs no initialization; calls that may overlap on the
  * GPU must use different scratch buffers. */
 
-/* The kernel soniq_mp_gemm runs for these arguments (SONIQ_PATH_*), or -1
+/* The path soniq_mp_gemm takes for these arguments (SONIQ_PATH_*), or -1
  * if it would return an error.  Host only (reads the device's SM count). */
 SONIQ_API int32_t soniq_mp_gemm_path(const soniq_layout *layout, int64_t M, int32_t N, uint32_t flags,
                                      size_t scratch_bytes);
+
+/* The kernel it runs (SONIQ_KERNEL_*), otherwise the same. */
+SONIQ_API int32_t soniq_mp_gemm_kernel(const soniq_layout *layout, int64_t M, int32_t N, uint32_t flags,
+                                       size_t scratch_bytes);
 
 /* Scratch bytes soniq_mp_gemm can use for these arguments (0: none).  Host
  * only; -1 on a bad argument. */

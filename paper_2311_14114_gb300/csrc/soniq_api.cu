@@ -212,7 +212,7 @@ size_t usable_scratch(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flag
     return optional && !aligned(scratch, 256) ? 0 : bytes;
 }
 
-// The kernel soniq_mp_gemm runs: a SONIQ_PATH_* value, -1 when the
+// The path soniq_mp_gemm takes: a SONIQ_PATH_* value, -1 when the
 // tensor-core kernel would be chosen but cannot take the layout (mma_check
 // says why), -2 when the GEMV was forced but cannot take the shape.
 int gemm_path(const LayoutGeom& geo, int64_t M, int32_t N, uint32_t flags, size_t scratch_bytes) {
@@ -222,8 +222,7 @@ int gemm_path(const LayoutGeom& geo, int64_t M, int32_t N, uint32_t flags, size_
         const int64_t need = staged_scratch_bytes(geo, M, N);
         return need > 0 && (int64_t)scratch_bytes >= need ? SONIQ_PATH_TENSOR_STAGED : -2;
     }
-    // up to SONIQ_GEMV_MAX_M rows the CUDA-core GEMV is faster; above, the tensor-core
-    // kernels (whose time hardly grows with M below 128) overtake it
+    // up to SONIQ_GEMV_MAX_M rows the GEMV's path, above that a tensor-core kernel
     const bool want_gemv =
         (flags & SONIQ_FLAG_FORCE_GEMV) ||
         (M <= SONIQ_GEMV_MAX_M && !(flags & (SONIQ_FLAG_FORCE_MMA | SONIQ_FLAG_FORCE_SKINNY)));
@@ -240,6 +239,16 @@ int gemm_path(const LayoutGeom& geo, int64_t M, int32_t N, uint32_t flags, size_
     }
     if (mma_check(geo) != SONIQ_OK) return -1;
     return SONIQ_PATH_TENSOR;
+}
+
+// Whether the calls of `path` run on warp-level tensor instructions (rows_mma.cu): from three
+// rows on, where the rows fit on chip and no flag asks for the GEMV or the swap-AB kernel
+// (11008 x 4096 at 3/6 bits, us, otherwise and so: M = 1 dot products 10.6 and 14.4; 2: 13.3, 14.7;
+// 4: 16.4, 14.7; 12: 37, 16; 16 swap-AB tcgen05 kernel 33.5, 16.7; 32: 37, 23; 4096 x 4096 4/8 bits:
+// M = 1 6.5, 7.5; 4: 8.2, 7.5; 16: 37, 8.9).
+bool takes_rows_kernel(const LayoutGeom& geo, int path, int64_t M, int64_t N, uint32_t flags) {
+    return (path == SONIQ_PATH_GEMV || path == SONIQ_PATH_TENSOR_SKINNY) && M >= 3 &&
+           !(flags & (SONIQ_FLAG_FORCE_GEMV | SONIQ_FLAG_FORCE_SKINNY)) && rows_mma_supported(geo, M, N);
 }
 
 // A per-tensor input of at most this many values is quantized by one CTA where its rows fit.
@@ -488,11 +497,7 @@ soniq_status soniq_mp_gemm(const soniq_layout* L, const uint8_t* Ap, const float
     if (path < 0) return path == -2 ? SONIQ_ERR_UNSUPPORTED : mma_check(geo);
     if (path == SONIQ_PATH_GEMV || path == SONIQ_PATH_TENSOR_SKINNY) {
         GemvArgs a{Ap, Wp, s_a, s_w, Y, acc_dbg, (int32_t)M, N, per_row, out_dtype == SONIQ_OUT_BF16};
-        // from three rows on, and where the rows fit on chip, warp-level tensor instructions
-        // (11008 x 4096 at 3/6 bits, us: M = 1 dot products 10.6 and 14.4; 2: 13.3, 14.7; 4: 16.4, 14.7;
-        // 12: 37, 16; 16 swap-AB tcgen05 kernel 33.5, 16.7; 32: 37, 23; 4096 x 4096 4/8 bits: M = 1 6.5, 7.5;
-        // 4: 8.2, 7.5; 16: 37, 8.9)
-        if (M >= 3 && rows_mma_supported(geo, M, N))
+        if (takes_rows_kernel(geo, path, M, N, flags))
             return cuda_status(launch_rows_mma(
                 geo, a, (flags & SONIQ_FLAG_TEST_DROP_ARRIVE) != 0 && path == SONIQ_PATH_TENSOR_SKINNY, s));
         if (path == SONIQ_PATH_GEMV) return cuda_status(launch_gemv(geo, a, s));
@@ -589,6 +594,13 @@ int32_t soniq_mp_gemm_path(const soniq_layout* L, int64_t M, int32_t N, uint32_t
     if ((flags & SONIQ_FLAG_FORCE_GEMV) && (flags & SONIQ_FLAG_FORCE_MMA)) return -1;
     const int p = gemm_path(geo, M, N, flags, scratch_bytes);
     return p < 0 ? -1 : p;
+}
+
+int32_t soniq_mp_gemm_kernel(const soniq_layout* L, int64_t M, int32_t N, uint32_t flags, size_t scratch_bytes) {
+    const int32_t path = soniq_mp_gemm_path(L, M, N, flags, scratch_bytes);
+    LayoutGeom geo;
+    if (path < 0 || make_geom(L, 1, &geo) != SONIQ_OK) return -1;
+    return takes_rows_kernel(geo, path, M, N, flags) ? SONIQ_KERNEL_ROWS : path;
 }
 
 int64_t soniq_mp_gemm_scratch_bytes(const soniq_layout* L, int64_t M, int32_t N, uint32_t flags) {

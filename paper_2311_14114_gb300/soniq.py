@@ -26,14 +26,17 @@ OUT_F16, OUT_BF16 = 0, 1
 FLAG_FORCE_GEMV, FLAG_FORCE_MMA, FLAG_FORCE_FUSED, FLAG_FORCE_STAGED = 1, 2, 4, 8
 FLAG_FORCE_SKINNY, FLAG_TEST_DROP_ARRIVE = 16, 0x100
 ACT_UNSIGNED, ACT_SIGNED, ACT_PM1 = 0, 1, 2
+# paths (soniq_mp_gemm_path) and the kernels behind them (soniq_mp_gemm_kernel)
 PATH_NAMES = {0: "CUDA-core GEMV", 1: "tensor-core fused kernel", 2: "tensor-core staged (expand + GEMM)",
-              3: "tensor-core skinny (swap-AB)"}
+              3: "tensor-core skinny"}
+KERNEL_NAMES = {0: "CUDA-core GEMV", 1: "tcgen05 fused", 2: "tcgen05 staged (expand + GEMM)", 3: "tcgen05 skinny (swap-AB)",
+                4: "warp-level tensor rows"}
 
 EXPORTED = ["soniq_abi_version", "soniq_status_string", "soniq_group_codes",
             "soniq_packed_row_bytes", "soniq_scale_runs", "soniq_validate_layout", "soniq_launch_count",
             "soniq_pack_weights", "soniq_quantize_act", "soniq_quantize_act_scratch_bytes",
-            "soniq_quantize_act_oneshot", "soniq_mp_gemm", "soniq_mp_gemm_path", "soniq_mp_gemm_scratch_bytes",
-            "soniq_mp_conv2d", "soniq_mp_conv2d_scratch_bytes", "soniq_sync_status",
+            "soniq_quantize_act_oneshot", "soniq_mp_gemm", "soniq_mp_gemm_path", "soniq_mp_gemm_kernel",
+            "soniq_mp_gemm_scratch_bytes", "soniq_mp_conv2d", "soniq_mp_conv2d_scratch_bytes", "soniq_sync_status",
             "soniq_test_drop_barrier_arrival"]
 
 _SCALE = {"tensor": SCALE_PER_TENSOR, "row": SCALE_PER_ROW, "calibrated": SCALE_CALIBRATED}
@@ -98,6 +101,8 @@ def lib() -> ctypes.CDLL:
         L.soniq_mp_gemm.restype = i32
         L.soniq_mp_gemm_path.argtypes = [P, i64, i32, u32, ctypes.c_size_t]
         L.soniq_mp_gemm_path.restype = i32
+        L.soniq_mp_gemm_kernel.argtypes = [P, i64, i32, u32, ctypes.c_size_t]
+        L.soniq_mp_gemm_kernel.restype = i32
         L.soniq_mp_gemm_scratch_bytes.argtypes = [P, i64, i32, u32]
         L.soniq_mp_gemm_scratch_bytes.restype = i64
         L.soniq_mp_conv2d.argtypes = [P, P, P, P, i32, P, P, P, i32, P, u32, P, ctypes.c_size_t, P, P]
@@ -341,13 +346,22 @@ def mp_gemm(layout: Layout, Ap: torch.Tensor, s_a: torch.Tensor, Wp: torch.Tenso
     return Y
 
 
-def gemm_path(layout: Layout, M: int, N: int, flags: int = 0) -> str:
-    """soniq_mp_gemm_path: the kernel soniq_mp_gemm runs for these arguments."""
+def _gemm_query(query, layout: Layout, M: int, N: int, flags: int) -> int:
     need = max(int(lib().soniq_mp_gemm_scratch_bytes(layout.ref, M, N, int(flags))), 0)
-    p = int(lib().soniq_mp_gemm_path(layout.ref, M, N, int(flags), need))
+    p = int(getattr(lib(), query)(layout.ref, M, N, int(flags), need))
     if p < 0:
-        raise SoniqError(SONIQ_ERR_INVALID_ARG, "soniq_mp_gemm_path")
-    return PATH_NAMES.get(p, str(p))
+        raise SoniqError(SONIQ_ERR_INVALID_ARG, query)
+    return p
+
+
+def gemm_path(layout: Layout, M: int, N: int, flags: int = 0) -> str:
+    """soniq_mp_gemm_path: the path soniq_mp_gemm takes for these arguments."""
+    return PATH_NAMES[_gemm_query("soniq_mp_gemm_path", layout, M, N, flags)]
+
+
+def gemm_kernel(layout: Layout, M: int, N: int, flags: int = 0) -> str:
+    """soniq_mp_gemm_kernel: the kernel soniq_mp_gemm runs for these arguments."""
+    return KERNEL_NAMES[_gemm_query("soniq_mp_gemm_kernel", layout, M, N, flags)]
 
 
 def conv_desc(batch, H, W, C_out, R=3, S=3, stride=(1, 1), pad=(1, 1)) -> CConvDesc:
