@@ -410,7 +410,7 @@ struct StreamParams {
 // One group of nr staged rows (row r's packed codes at src), by one warp of wpr: its
 // pieces are those of index sub modulo wpr, 32 at a time.  sum: wpr > 1, the shared
 // word of the row's and group's code sum.
-template <int N, int PARTS>
+template <int N, int PARTS, bool LONG>
 __device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src, int64_t r, int nr, int g, int lane, int sub,
                                              int wpr, int32_t* sum) {
     const bool vec8 = p.vec8[g] != 0;
@@ -423,7 +423,7 @@ __device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src
     for (int i = 0; i < nr; ++i, src += (uint32_t)p.src_row_bytes, drow += p.dst_row_bytes) {
         int32_t csum = 0;
 #pragma unroll 2
-        for (int c = lane + 32 * sub; c < pieces; c += 32 * wpr) {
+        for (int c = LONG ? lane + 32 * sub : lane; c < pieces; c += LONG ? 32 * wpr : 32) {
             const int kb = c / PARTS, part = c % PARTS;
             PartWords<N, PARTS> w;
             if (c < have) w.load(SharedWords{src + (uint32_t)(kb * 4 * N)}, part, vec8);
@@ -433,13 +433,16 @@ __device__ __forceinline__ void stream_group(const ExpandParams& p, uint32_t src
         if (PARTS == 4 && p.is_weight) {
             const int32_t s = __reduce_add_sync(0xffffffffu, csum);
             if (lane == 0) {
-                if (wpr == 1) p.colsum[(r + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
+                if (!LONG || wpr == 1) p.colsum[(r + i) * 2 + g] = s - (1 << (N - 1)) * 32 * p.blk_dst[g];
                 else atomicAdd(sum, s);
             }
         }
     }
 }
 
+// LONG: rows shared by warps, or tiles off the 16-byte grid (the general form, whose run-time
+// strides cost the others 3 to 13 %).
+template <bool LONG>
 __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kernel(const __grid_constant__ StreamParams sp) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full_bar[kStreamMaxStages], empty_bar[kStreamMaxStages];
@@ -456,11 +459,11 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
         none_s = 0u;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (threadIdx.x < kStreamMaxStages * kStreamWarps) (&sums_s[0][0])[threadIdx.x] = 0;
+    if (LONG && threadIdx.x < kStreamMaxStages * kStreamWarps) (&sums_s[0][0])[threadIdx.x] = 0;
     __syncthreads();
     tc::pdl_wait();      // launched with launch_pdl: the packed rows are written before this
     // (no early trigger: GEMM CTAs that move in as this kernel's leave cost the MLP block 14 us)
-    const int tr = kStreamWarps / sp.wpr * sp.rpw;         // rows per tile
+    const int wpr = LONG ? sp.wpr : 1, tr = kStreamWarps / wpr * sp.rpw;         // warps per row, rows per tile
     const int64_t tiles_a = (sp.op[0].rows + tr - 1) / tr;
     const int64_t tiles = tiles_a + (sp.op[1].rows + tr - 1) / tr;
     int b = 0;
@@ -484,7 +487,7 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
             if (issued >= sp.stages) {
                 ok = tc::wait_bounded_warp(tc::smem_u32(&empty_bar[b]), ph ^ 1u, abort_flag, kTimeoutNs, sp.err, kErrWait);
                 if (!ok) break;
-                if (sp.wpr > 1) flush(t - behind, b);
+                if (LONG && wpr > 1) flush(t - behind, b);
             }
             const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
             const int64_t r0 = (t < tiles_a ? t : t - tiles_a) * tr;
@@ -492,7 +495,7 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
             // the tile keeps its global address modulo 16: one bulk copy of the aligned interior,
             // lanes 0..2 move the words before it, 4..6 those after it
             const uint8_t* src = p.src + r0 * p.src_row_bytes;
-            const int shift = (int)((uintptr_t)src & 15u), bytes = nr * (int)p.src_row_bytes;
+            const int shift = LONG ? (int)((uintptr_t)src & 15u) : 0, bytes = nr * (int)p.src_row_bytes;
             const int head = min((16 - shift) & 15, bytes), body = (bytes - head) & ~15, tail = bytes - head - body;
             const uint32_t dst = base + (uint32_t)(b * sp.stage_bytes + shift), bar = tc::smem_u32(&full_bar[b]);
             if (lane == 0 && body > 0) {
@@ -511,7 +514,7 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
                 ph ^= 1u;
             }
         }
-        if (ok && sp.wpr > 1) {
+        if (LONG && ok && wpr > 1) {
             // the code sums still in the ring
             for (int64_t i = issued > sp.stages ? issued - sp.stages : 0; i < issued && ok; ++i) {
                 const int st = (int)(i % sp.stages);
@@ -528,24 +531,24 @@ __global__ void __launch_bounds__((kStreamWarps + 1) * 32, 4) expand_stream_kern
         return;
     }
     // ---- consumers: warp -> rows row0 .. row0 + rpw - 1 of a tile, pieces sub modulo wpr ----
-    const int row0 = warp / sp.wpr * sp.rpw, sub = warp % sp.wpr;
+    const int row0 = warp / wpr * sp.rpw, sub = warp % wpr;
     for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
         if (!tc::wait_bounded_warp(tc::smem_u32(&full_bar[b]), ph, abort_flag, kTimeoutNs, sp.err, kErrWait)) return;
         const ExpandParams& p = sp.op[t < tiles_a ? 0 : 1];
         const int64_t r0 = (t < tiles_a ? t : t - tiles_a) * tr, r = r0 + row0;
         const int nr = p.rows - r < sp.rpw ? (int)(p.rows - r) : sp.rpw;
         if (nr > 0) {
-            uint32_t row = base + (uint32_t)(b * sp.stage_bytes) + ((uint32_t)(uintptr_t)(p.src + r0 * p.src_row_bytes) & 15u) +
-                           (uint32_t)(row0 * (int)p.src_row_bytes);
+            uint32_t row = base + (uint32_t)(b * sp.stage_bytes) + (uint32_t)(row0 * (int)p.src_row_bytes);
+            if (LONG) row += (uint32_t)(uintptr_t)(p.src + r0 * p.src_row_bytes) & 15u;
             asm volatile("" : "+r"(row)::"memory");        // keeps the row's loads behind the wait
 #pragma unroll 1
             for (int g = 0; g < 2; ++g) {
                 if (p.blk_dst[g] == 0) continue;
                 const uint32_t src = row + (uint32_t)p.src_off[g];
                 const int n = p.bits[g];
-                int32_t* sum = &sums_s[b][2 * (warp / sp.wpr) % kStreamWarps + g];
+                int32_t* sum = &sums_s[b][2 * (warp / wpr) % kStreamWarps + g];
                 auto group = [&](auto bits, auto parts) {
-                    stream_group<decltype(bits)::value, decltype(parts)::value>(p, src, r, nr, g, lane, sub, sp.wpr, sum);
+                    stream_group<decltype(bits)::value, decltype(parts)::value, LONG>(p, src, r, nr, g, lane, sub, wpr, sum);
                 };
                 using std::integral_constant;
                 constexpr integral_constant<int, 1> c1{};
@@ -621,18 +624,19 @@ bool launch_stream(const ExpandParams& a, const ExpandParams& w, cudaStream_t st
     sp.rpw = (int32_t)rpw;
     sp.wpr = (int32_t)wpr;
     const int64_t tiles = (a.rows + tr - 1) / tr + (w.rows + tr - 1) / tr;
-    static bool attr_done[64] = {};
+    const bool is_long = wpr > 1 || !grid16;
+    const auto fn = is_long ? expand_stream_kernel<true> : expand_stream_kernel<false>;
+    static bool attr_done[64][2] = {};
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) return false;
-    if (!attr_done[dev]) {
-        *err = cudaFuncSetAttribute(expand_stream_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)kStreamSmemPerSm);
-        if (*err == cudaSuccess) *err = prefer_max_shared((const void*)expand_stream_kernel);
+    if (!attr_done[dev][is_long]) {
+        *err = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kStreamSmemPerSm);
+        if (*err == cudaSuccess) *err = prefer_max_shared((const void*)fn);
         if (*err != cudaSuccess) return true;
-        attr_done[dev] = true;
+        attr_done[dev][is_long] = true;
     }
-    *err = launch_pdl(expand_stream_kernel, dim3((unsigned)(tiles < cap ? tiles : cap)), dim3((kStreamWarps + 1) * 32),
+    *err = launch_pdl(fn, dim3((unsigned)(tiles < cap ? tiles : cap)), dim3((kStreamWarps + 1) * 32),
                       (size_t)(sp.stages * sp.stage_bytes), st, sp);
     return true;
 }
