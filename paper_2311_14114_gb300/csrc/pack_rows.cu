@@ -142,15 +142,16 @@ __global__ void __launch_bounds__((WARPS + 1) * 32, CTAS) pack_rows_kernel(const
                 ++round;
             }
         }
-        if (!ok && lane == 0) {
-            // abandoned: the copies in flight land before the CTA exits (the abort flag is up, so
-            // each wait gets a flag of its own)
+        if (lane == 0) {
+            // the copies in flight land before the CTA exits, also when it was abandoned (the abort
+            // flag may be up, so these waits get a flag of their own)
             __shared__ uint32_t none_s;
             none_s = 0u;
             for (int i = 0; i < p.stages; ++i) {
-                const uint32_t ph = i < b ? round : round - 1u;
-                tc::wait_bounded(tc::smem_u32(&full_bar[i]), ph & 1u, tc::smem_u32(&none_s), p.timeout_ns, p.err,
-                                 kErrWait);
+                const uint32_t uses = round + (i < b ? 1u : 0u);        // tiles the stage has taken
+                if (uses > 0u)
+                    tc::wait_bounded(tc::smem_u32(&full_bar[i]), (uses - 1u) & 1u, tc::smem_u32(&none_s), p.timeout_ns,
+                                     p.err, kErrWait);
             }
         }
         return;

@@ -237,7 +237,7 @@ template <int MODE>
 __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(const GatherParams p) {
     extern __shared__ __align__(128) uint8_t smem[];
     __shared__ __align__(8) uint64_t full_bar[kGatherMaxStages], empty_bar[kGatherMaxStages];
-    __shared__ uint32_t abort_s, lost_s, max_s[2];
+    __shared__ uint32_t abort_s, none_s, lost_s, max_s[2];
     __shared__ GConst kc_s[2][kGatherMaxRows][2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int TR = p.tile_rows, NST = p.stages, K = p.K;
@@ -304,6 +304,15 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
                     b = 0;
                     ++round;
                 }
+            }
+            // the copies in flight land before the CTA exits, also when it was abandoned (the abort
+            // flag may be up, so these waits get a flag of their own)
+            none_s = 0u;
+            for (int i = 0; i < NST; ++i) {
+                const uint32_t taken = round + (i < b ? 1u : 0u);       // tiles the stage has taken
+                if (taken > 0u)
+                    tc::wait_bounded(tc::smem_u32(&full_bar[i]), (taken - 1u) & 1u, tc::smem_u32(&none_s), p.timeout_ns,
+                                     p.err, kErrWait);
             }
         }
         return;
