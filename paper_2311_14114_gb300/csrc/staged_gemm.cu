@@ -79,7 +79,7 @@ constexpr int NUM_EPI_WARPS = 8;
 constexpr int WARP_TMA = 0, WARP_MMA = 1, WARP_EPI = 4;      // warps 2 and 3 only give up registers
 constexpr int NUM_THREADS = (WARP_EPI + NUM_EPI_WARPS) * 32;
 
-// Epilogues.  LEAN, SEG, NEXT and RUNS read the accumulators as MMA fragments
+// Epilogues.  LEAN, SEG, NEXT, NEXT_SEG and RUNS read the accumulators as MMA fragments
 // (fragment epilogue below); GENERAL and GENERAL_NEXT, one row per lane, also
 // write debug accumulators.
 enum {
@@ -87,9 +87,15 @@ enum {
     EPI_SEG = 1,           // one group in exact segments, drained to int32
     EPI_NEXT = 2,          // LEAN, plus the next layer's codes (quantize-in-epilogue)
     EPI_RUNS = 3,          // scale runs along K
-    EPI_GENERAL = 4,
-    EPI_GENERAL_NEXT = 5
+    EPI_NEXT_SEG = 4,      // NEXT with one group in exact segments
+    EPI_GENERAL = 5,
+    EPI_GENERAL_NEXT = 6
 };
+
+template <int EPI>
+constexpr bool kEpiSegments = EPI == EPI_SEG || EPI == EPI_NEXT_SEG;
+template <int EPI>
+constexpr bool kEpiNext = EPI == EPI_NEXT || EPI == EPI_NEXT_SEG;
 
 // How outputs leave: OUT_BATCH stages 32 rows x 32 columns per epilogue warp
 // (2 KB) at a time and copies them out with 16-byte stores, which leaves the
@@ -991,7 +997,7 @@ struct ColPlan {
     int centf, centl;          // centring of group f / l (0: none)
     float saf, sal;            // per-tensor activation scales (1: per row)
     __device__ __forceinline__ explicit ColPlan(const SParams& p) {
-        gA = EPI == EPI_SEG ? first_group(p) : 0;      // in segments only group gA may be
+        gA = kEpiSegments<EPI> ? first_group(p) : 0;   // in segments only group gA may be
         const int gB = 1 - gA;
         nA = p.g[gA].stages > 0 ? p.g[gA].n_seg : 0;
         const int nB = p.g[gB].stages > 0 ? p.g[gB].n_seg : 0;
@@ -999,7 +1005,7 @@ struct ColPlan {
         gl = nB > 0 ? gB : gA;
         gf = 1 - gl;
         both = nA > 0 && nB > 0;
-        same = EPI == EPI_SEG && !both;
+        same = kEpiSegments<EPI> && !both;
         invf = p.g[gf].inv_levels;
         invl = p.g[gl].inv_levels;
         scf = p.g[gf].acc_scale;
@@ -1040,7 +1046,7 @@ struct ColLoad {
             d[2] = __fmul_rn(cp.sal, (cp.gl ? sw.y : sw.x) * cp.invl);
             // int32 where the group's sum is one, else fp32 (exact)
             const int f = cp.centf * cf, l = cp.centl * cl;
-            d[4] = EPI == EPI_SEG ? __int_as_float(f) : (float)f;
+            d[4] = kEpiSegments<EPI> ? __int_as_float(f) : (float)f;
             d[6] = cp.same ? __int_as_float(l) : (float)l;
         }
         __syncwarp();
@@ -1057,7 +1063,7 @@ __device__ __forceinline__ bool frag_tile(const SParams& p, const ColPlan<EPI>& 
                                           ColLoad& cl, uint32_t& job, Release&& release) {
     using C = Cfg<BNT, PAIR, OUT>;
     constexpr int EPI_COLS = C::EPI_COLS, NCH = EPI_COLS / 8;
-    constexpr bool SEG = EPI == EPI_SEG, NEXT = EPI == EPI_NEXT;
+    constexpr bool SEG = kEpiSegments<EPI>, NEXT = kEpiNext<EPI>;
     const int lane = t.lane;
     auto wait = [&](int b, uint32_t ph) {
         return __all_sync(0xffffffffu, wait_bounded(t.bar0 + 8u * (uint32_t)b, ph, t.abort_flag, kTimeoutNs, p.err,
@@ -1299,7 +1305,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
     constexpr int BN = BNT;
     constexpr int STAGE_BYTES = C::STAGE_BYTES, STAGES = C::STAGES, EPI_COLS = C::EPI_COLS;
     constexpr int COLS_BYTES = C::COLS_BYTES, OUT_PER_WARP = C::OUT_PER_WARP;
-    static_assert((EPI >= EPI_GENERAL) == (OUT == OUT_GENERAL) && (EPI != EPI_NEXT || OUT == OUT_TMA), "epilogue and outputs");
+    static_assert((EPI >= EPI_GENERAL) == (OUT == OUT_GENERAL) && (!kEpiNext<EPI> || OUT == OUT_TMA), "epilogue and outputs");
     constexpr int BAR_FULL = C::BAR_FULL, BAR_EMPTY = C::BAR_EMPTY, BAR_REG_FULL = C::BAR_REG_FULL,
                   BAR_REG_EMPTY = C::BAR_REG_EMPTY, BAR_TEARDOWN = C::BAR_TEARDOWN;
     constexpr int SMEM_OUT = C::SMEM_OUT, SMEM_COLS = C::SMEM_COLS, SMEM_BAR = C::SMEM_BAR, SMEM_MISC = C::SMEM_MISC;
@@ -1825,8 +1831,9 @@ const Variant kVariants[] = {
     make_variant<EPI_SEG, true, 256, true, OUT_BATCH>(),    make_variant<EPI_SEG, true, 256, false, OUT_BATCH>(),
     make_variant<EPI_SEG, true, 128, false, OUT_BATCH>(),   make_variant<EPI_SEG, true, 240, true, OUT_BATCH>(),
     make_variant<EPI_SEG, true, 240, false, OUT_BATCH>(),   make_variant<EPI_NEXT, false, 256, false, OUT_TMA>(),
-    make_variant<EPI_NEXT, true, 256, false, OUT_TMA>(),    make_variant<EPI_RUNS, false, 128, false, OUT_BATCH>(),
-    make_variant<EPI_RUNS, false, 64, false, OUT_BATCH>(),  make_variant<EPI_RUNS, true, 64, false, OUT_BATCH>(),   make_variant<EPI_GENERAL, true, 256, false, OUT_GENERAL>(),
+    make_variant<EPI_NEXT, true, 256, false, OUT_TMA>(),    make_variant<EPI_NEXT_SEG, true, 256, false, OUT_TMA>(),
+    make_variant<EPI_RUNS, false, 128, false, OUT_BATCH>(), make_variant<EPI_RUNS, false, 64, false, OUT_BATCH>(),
+    make_variant<EPI_RUNS, true, 64, false, OUT_BATCH>(),   make_variant<EPI_GENERAL, true, 256, false, OUT_GENERAL>(),
     make_variant<EPI_GENERAL, true, 240, false, OUT_GENERAL>(),
     make_variant<EPI_GENERAL_NEXT, true, 256, false, OUT_GENERAL>(),
 };
@@ -2038,10 +2045,10 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     // ---- epilogue, tile width and pairing ----
     const bool runs = geo.sub_k > 0, wr_y = a.Y != nullptr, has_next = a.next != nullptr;
     const bool general = !runs && (a.acc_dbg != nullptr || (!wr_y && !has_next) ||
-                                   (a.flags & SONIQ_FLAG_TEST_DROP_ARRIVE) != 0 || (has_next && sp.seg_group >= 0));
+                                   (a.flags & SONIQ_FLAG_TEST_DROP_ARRIVE) != 0);
     const int epi = runs ? EPI_RUNS
                     : general ? (has_next ? EPI_GENERAL_NEXT : EPI_GENERAL)
-                    : has_next ? EPI_NEXT
+                    : has_next ? (sp.seg_group >= 0 ? EPI_NEXT_SEG : EPI_NEXT)
                     : sp.seg_group >= 0 ? EPI_SEG : EPI_LEAN;
     const Variant* var = pick_variant(epi, runs ? a.acc_dbg != nullptr : a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0, a.M, a.N, (int)(sp.eb / KSTAGE));
     if (var == nullptr) return cudaErrorNotSupported;
