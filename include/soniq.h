@@ -135,7 +135,8 @@ enum {
     SONIQ_FLAG_FORCE_STAGED = 8u,        /* tensor-core work takes the staged path whenever the
                                             scratch suffices, however small the problem (without
                                             it the staged path is used from 2^30 multiply-adds
-                                            on, and for most smaller calls with long rows) */
+                                            on, and for most smaller calls with long rows and
+                                            no acc_dbg) */
     SONIQ_FLAG_FORCE_SKINNY = 16u,       /* tensor-core work takes the skinny swap-AB kernel
                                             (M <= 32, taps = 1, groups padded to 128 codes) */
     SONIQ_FLAG_TEST_DROP_ARRIVE = 0x100u /* test hook: the tensor-core kernels' operand producer
@@ -381,8 +382,8 @@ SONIQ_API soniq_status soniq_mp_gemm(const soniq_layout *layout, const uint8_t *
  * bits.  The scratch needs no initialization; calls that may overlap on the
  * GPU must use different scratch buffers. */
 
-/* The path soniq_mp_gemm takes for these arguments (SONIQ_PATH_*), or -1
- * if it would return an error.  Host only (reads the device's SM count). */
+/* The path soniq_mp_gemm takes for these arguments without acc_dbg (SONIQ_PATH_*),
+ * or -1 if it would return an error.  Host only (reads the device's SM count). */
 SONIQ_API int32_t soniq_mp_gemm_path(const soniq_layout *layout, int64_t M, int32_t N, uint32_t flags,
                                      size_t scratch_bytes);
 

@@ -204,12 +204,14 @@ bool staged_worthwhile(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t fla
 
 // The scratch bytes a call may use.  Scratch off the 256-byte grid is an error where only
 // the staged path will do (forced, a layout variant) or from 2^30 multiply-adds on; smaller
-// calls run without it.
-size_t usable_scratch(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flags, const void* scratch, size_t bytes) {
+// calls run without it, as do smaller calls with debug accumulators, whose staged epilogue is
+// slow (655 x 512 x 2368 with them: fused 40 us, staged 71; 2423 x 384 x 64 19, 29).
+size_t usable_scratch(const LayoutGeom& geo, int64_t M, int64_t N, uint32_t flags, const void* acc_dbg, const void* scratch,
+                      size_t bytes) {
     if (scratch == nullptr) return 0;
     const bool optional = !geo.variant && !(flags & SONIQ_FLAG_FORCE_STAGED) &&
                           (double)M * (double)N * (double)geo.K * (double)geo.taps < 1073741824.0;
-    return optional && !aligned(scratch, 256) ? 0 : bytes;
+    return optional && (acc_dbg != nullptr || !aligned(scratch, 256)) ? 0 : bytes;
 }
 
 // The path soniq_mp_gemm takes: a SONIQ_PATH_* value, -1 when the
@@ -492,7 +494,7 @@ soniq_status soniq_mp_gemm(const soniq_layout* L, const uint8_t* Ap, const float
     if (next != nullptr)
         flags = (flags & ~(uint32_t)(SONIQ_FLAG_FORCE_GEMV | SONIQ_FLAG_FORCE_SKINNY)) | SONIQ_FLAG_FORCE_MMA |
                 SONIQ_FLAG_FORCE_STAGED;
-    const int path = gemm_path(geo, M, N, flags, usable_scratch(geo, M, N, flags, scratch, scratch_bytes));
+    const int path = gemm_path(geo, M, N, flags, usable_scratch(geo, M, N, flags, acc_dbg, scratch, scratch_bytes));
     if (next != nullptr && path != SONIQ_PATH_TENSOR_STAGED) return SONIQ_ERR_UNSUPPORTED;
     if (path < 0) return path == -2 ? SONIQ_ERR_UNSUPPORTED : mma_check(geo);
     if (path == SONIQ_PATH_GEMV || path == SONIQ_PATH_TENSOR_SKINNY) {
@@ -549,7 +551,7 @@ soniq_status soniq_mp_conv2d(const soniq_layout* L, const soniq_conv_desc* cd, c
     if (!aligned(Xp, 4) || !aligned(Wp, 16) || !aligned(Y, 16) || !aligned(s_a, 4) || !aligned(s_w, 4) ||
         (acc_dbg != nullptr && !aligned(acc_dbg, 4)))
         return SONIQ_ERR_ALIGNMENT;
-    scratch_bytes = usable_scratch(geo, M, cd->C_out, flags, scratch, scratch_bytes);
+    scratch_bytes = usable_scratch(geo, M, cd->C_out, flags, acc_dbg, scratch, scratch_bytes);
     const bool staged = !(flags & SONIQ_FLAG_FORCE_FUSED) && staged_worthwhile(geo, M, cd->C_out, flags) &&
                         staged_scratch_bytes(geo, M, cd->C_out) > 0 &&
                         (int64_t)scratch_bytes >= staged_scratch_bytes(geo, M, cd->C_out);
