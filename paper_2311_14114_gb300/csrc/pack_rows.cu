@@ -298,6 +298,10 @@ cudaError_t launch_pack_rows(const LayoutGeom& geo, const int32_t* perm, const f
     const int64_t L = (int64_t)geo.taps * geo.K;
     const int nblk0 = geo.g[0].pw / 32, nblk1 = geo.g[1].pw / 32;
     if (L > 32768 || nblk0 + nblk1 == 0) return cudaErrorNotSupported;
+    // A few short rows of one group are one warp's work either way, and staging them only adds to
+    // it: a CTA per row of the plain kernel is as quick or quicker (us, plain and staged: 33 x 128
+    // 2.7, 3.7; 162 x 128 2.9, 4.1; 162 x 79 2.9, 3.5; 645 x 128 3.1, 3.2; 2000 x 128 4.9, 3.3).
+    if (nblk0 + nblk1 == 4 && L <= 128 && N <= 192) return cudaErrorNotSupported;
     PackRowsParams p;
     p.W = W;
     p.Wp = Wp;
