@@ -547,12 +547,6 @@ __global__ void __launch_bounds__(kGatherThreads, 1) quantize_gather_kernel(cons
 
 }  // namespace
 
-// Tiled quantize with bulk-staged rows (quantize_gather_kernel).  Needs rows
-// of 16-byte-aligned 16-byte multiples (K % 8 == 0, A 16-byte aligned) and
-// room for at least one row per stage; returns cudaErrorNotSupported
-// otherwise.  scale_mode PER_ROW finds the scales; the others read s_a[2].
-// demote: the input's L2 lines were read with an evict-last policy (the
-// absmax pass), and their priority is reset as they are read here.
 namespace {
 
 struct GatherPlan {

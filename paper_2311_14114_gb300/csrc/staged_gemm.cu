@@ -1543,14 +1543,14 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
         // ------------------------------------------------------------- epilogue
         asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
         // Warp w reads TMEM lane quadrant w % 4 (rows 32*(w%4) .. +31 of the
-        // tile) and the 128 columns cgrp*128 .. +127, cgrp = (w - 2) / 4.
+        // tile) and the EPI_COLS columns from cgrp * EPI_COLS, cgrp = (w - 4) / 4.
         const int ew = warp - WARP_EPI;
         const int quad = warp & 3;
         const int cgrp = ew >> 2;
         const int row = quad * 32 + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(cgrp * EPI_COLS);
-        // this warp's copy of the tile's column constants: {s_w0 * inv_levels0,
-        // s_w1 * inv_levels1, center0 * C0, center1 * C1} per column
+        // column constants (GENERAL: this warp's copy, per column {s_w0 * inv_levels0,
+        // s_w1 * inv_levels1, center0 * C0, center1 * C1}; the others: FragTile::colc)
         float4* colc = reinterpret_cast<float4*>(smem + SMEM_COLS + ew * COLS_BYTES);
         const uint32_t out_s = sbase + (uint32_t)(SMEM_OUT + ew * OUT_PER_WARP);   // 1024-aligned
         // a drained TMEM region goes back to the CTA that issues the MMAs
@@ -1754,7 +1754,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) staged_mma_kernel(const __grid
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // the peer multicasts into this CTA's stages and arrives on its barriers until it is done
+    // the peer's MMAs read this CTA's stages and its commits arrive on this CTA's barriers until it is done
     if constexpr (PAIR) cluster_sync();
     if (warp == WARP_MMA) {
         if constexpr (PAIR)
@@ -1805,7 +1805,7 @@ bool encode_rows(EncodeTiledFn enc, CUtensorMap* map, const uint8_t* base, int64
 
 struct Variant {
     int epi;
-    bool rows;       // activation scales per row (LEAN, NEXT); debug accumulators (RUNS)
+    bool rows;       // LEAN, NEXT: activation scales per row; RUNS: writes debug accumulators (runs_tile's DBG)
     bool f4;
     int bn;
     bool pair;
@@ -1844,7 +1844,8 @@ constexpr int kNumVariants = (int)(sizeof(kVariants) / sizeof(kVariants[0]));
 // 256 TMA 132, 128 156, 64 259; 16384 x 768 x 3072 pair 82, 256 73, 256 TMA 66, 128 79,
 // 64 117; 2048 x 4096 x 11008 pair 83, 256 92, 128 116; 512 x 4096 x 4096 pair 28, 256 26,
 // 128 23, 64 31; 300 x 4096 x 1024 pair 23, 256 21, 128 17, 64 16.  (An MMA takes about 110
-// cycles however narrow, so 64 columns pay only where 128 leave SMs idle.)
+// cycles however narrow, so 64 columns pay only where 128 leave SMs idle.)  There is no term of
+// its own for a scale run's drain or for E2M1 stages: those layouts choose by the same costs, unfitted.
 struct TileCost {
     double stage, fixed, epilogue;
 };
@@ -1973,7 +1974,6 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     uint8_t* xa = static_cast<uint8_t*>(scratch);
     uint8_t* xw = xa + align1k(rows_a * sp.eb);
     int32_t* colsum = reinterpret_cast<int32_t*>(xw + align1k((int64_t)a.N * sp.eb));
-    const int taps = a.conv ? a.R * a.S : 1;
 
     // ---- expand activations (im2col for a convolution) and weights ----
     ExpandParams e;
@@ -2004,7 +2004,6 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
     e.conv = a.conv;
     e.H = a.H; e.W = a.W; e.P = a.P; e.Q = a.Q; e.R = a.R; e.S = a.S;
     e.sh = a.sh; e.sw = a.sw; e.ph = a.ph; e.pw = a.pw;
-    (void)taps;
     auto grid_for = [](int64_t items) {
         int64_t ctas = (items + 7) / 8;                        // 8 warps per CTA, one (four rows, group) per warp
         const int64_t cap = (int64_t)num_sms() * 16;
@@ -2050,7 +2049,8 @@ cudaError_t launch_staged(const LayoutGeom& geo, const MmaArgs& a, void* scratch
                     : general ? (has_next ? EPI_GENERAL_NEXT : EPI_GENERAL)
                     : has_next ? (sp.seg_group >= 0 ? EPI_NEXT_SEG : EPI_NEXT)
                     : sp.seg_group >= 0 ? EPI_SEG : EPI_LEAN;
-    const Variant* var = pick_variant(epi, runs ? a.acc_dbg != nullptr : a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0, a.M, a.N, (int)(sp.eb / KSTAGE));
+    const Variant* var = pick_variant(epi, runs ? a.acc_dbg != nullptr : a.s_a_per_row != 0, sp.f4 != 0, wr_y && a.N % 8 == 0,
+                                      a.M, a.N, (int)(sp.eb / KSTAGE));
     if (var == nullptr) return cudaErrorNotSupported;
     const int tile_n = var->bn;
     const bool pair = var->pair;
