@@ -7,7 +7,6 @@ no GPU is present the calls raise.
 """
 from __future__ import annotations
 
-import contextlib
 import ctypes
 import os
 from typing import Optional, Sequence, Tuple
@@ -160,12 +159,19 @@ def _need(t: torch.Tensor, dtype, name: str):
 _scratch = {}
 
 
+def _graph_scratch(nbytes: int, device, use: str) -> torch.Tensor:
+    return (torch.zeros if use == "quantize" else torch.empty)(nbytes, dtype=torch.uint8, device=device)
+
+
 def _get_scratch(nbytes: int, device, stream, use: str) -> Optional[torch.Tensor]:
     if nbytes <= 0:
         return None
-    with contextlib.nullcontext() if stream is None else torch.cuda.stream(stream):
-        if torch.cuda.is_current_stream_capturing():
-            return (torch.zeros if use == "quantize" else torch.empty)(nbytes, dtype=torch.uint8, device=device)
+    if stream is not None:
+        with torch.cuda.stream(stream):
+            if torch.cuda.is_current_stream_capturing():
+                return _graph_scratch(nbytes, device, use)
+    elif torch.cuda.is_current_stream_capturing():
+        return _graph_scratch(nbytes, device, use)
     index = device.index
     key = (use, index, _current(index) if stream is None else stream.cuda_stream)
     buf = _scratch.get(key)
