@@ -433,8 +433,9 @@ SONIQ_API int64_t soniq_mp_conv2d_scratch_bytes(const soniq_layout *layout, cons
 SONIQ_API soniq_status soniq_sync_status(soniq_stream_t stream);
 
 /* Test hook, not for production use.  When armed (armed != 0), the next
- * launch of the one-pass per-tensor quantize kernel, from soniq_quantize_act
- * or soniq_quantize_act_oneshot, has its first CTA skip its grid-barrier
+ * launch of a per-tensor quantize kernel with a grid barrier (one-pass or
+ * streamed), from soniq_quantize_act or soniq_quantize_act_oneshot, has its
+ * first CTA skip its grid-barrier
  * arrival: the other CTAs' bounded waits run out after 2 s, the outputs are
  * not written, and soniq_sync_status reports SONIQ_ERR_TIMEOUT.  The hook
  * disarms itself at that launch.  No fault, trap or hang is involved. */
